@@ -313,7 +313,6 @@ fw_status plan_build(fw_batched_plan* p) {
     a.n = p->n[g];
     a.ld = p->ld[g];
     a.R = p->R[g];
-    a.slot_tiles = w.slot_tiles;
     a.ver = reinterpret_cast<int*>(base + flag_off[g]);
     a.done = a.ver + (size_t)p->R[g] * p->R[g];
     a.ctr = reinterpret_cast<unsigned*>(a.done + 2 * (size_t)p->R[g]);
@@ -324,15 +323,7 @@ fw_status plan_build(fw_batched_plan* p) {
     a.skip_task = -1;
     a.timeout_ns = p->opt.timeout_ns > 0 ? p->opt.timeout_ns : 2000000000LL;
     a.packed = p->opt.packed_keys ? 1 : 0;
-    a.piv = reinterpret_cast<T*>(w.piv);
-    a.pivP = w.pivP;
-    a.colK = w.colK;
-    a.colR = reinterpret_cast<T*>(w.colR);
-    a.colB = w.colB;
-    a.rowK = w.rowK;
-    a.rowR = reinterpret_cast<T*>(w.rowR);
-    a.rowP = w.rowP;
-    a.rowB = w.rowB;
+    fwk::set_snapshots(a, w);
     a.trace = nullptr;
     ha[g] = a;
     if (cudaMemcpy(w.stage_off, offs[g].data(), offs[g].size() * 4, cudaMemcpyHostToDevice) !=

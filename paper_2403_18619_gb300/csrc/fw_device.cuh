@@ -187,6 +187,33 @@ __device__ __forceinline__ void stamp(int i) {
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
 }
+__device__ __forceinline__ void mbar_arrive_n(uint64_t* bar, unsigned count) {
+  asm volatile("mbarrier.arrive.shared.b64 _, [%0], %1;" ::"r"(smem_u32(bar)), "r"(count)
+               : "memory");
+}
+
+// Predicated stores: no branch around a store that few lanes make, so that the
+// work of the entries around it overlaps.
+__device__ __forceinline__ void st_if(bool p, int32_t* a, int32_t v) {
+  asm volatile("{\n .reg .pred p;\n setp.ne.u32 p, %0, 0;\n @p st.global.b32 [%1], %2;\n}" ::"r"(
+                   (unsigned)p),
+               "l"(a), "r"(v)
+               : "memory");
+}
+__device__ __forceinline__ void st_if(bool p, int32_t* a, const int32_t (&v)[4]) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %0, 0;\n @p st.global.v4.b32 [%1], {%2, %3, %4, %5};\n}" ::
+          "r"((unsigned)p),
+      "l"(a), "r"(v[0]), "r"(v[1]), "r"(v[2]), "r"(v[3])
+      : "memory");
+}
+__device__ __forceinline__ void st_if(bool p, int32_t* a, const int32_t (&v)[2]) {
+  asm volatile(
+      "{\n .reg .pred p;\n setp.ne.u32 p, %0, 0;\n @p st.global.v2.b32 [%1], {%2, %3};\n}" ::"r"(
+          (unsigned)p),
+      "l"(a), "r"(v[0]), "r"(v[1])
+      : "memory");
+}
 
 // ------------------------------------------------------------- geometry ----
 
@@ -223,6 +250,43 @@ struct Keys {
   static constexpr int CAP = (1 << (31 - KB)) - 1;
   static_assert((1 << (KB - 1)) == BS, "BS must be 32, 64 or 128");
 };
+
+// 16-bit packed keys, two steps of the k loop per 32-bit word: a word of an
+// operand row holds the keys of steps kk_lo (low half) and kk_hi (high half),
+// so that one __viaddmin_u16x2 relaxes an output through both.  A key is
+// d << KB | kk (operand A; B without kk): the smaller half of an accumulator
+// is the smallest sum, reached first at its kk.
+//   kCapF bounds tiles without a missing edge: the sums of two operands stay
+//         below it;
+//   kCapI is INF where an operand has a missing edge: two of them do not wrap.
+template <int BS>
+struct KeysH {
+  static constexpr int kNW = BS / 32;                   // words per thread and operand row
+  static constexpr int KB = (BS == 128) ? 7 : (BS == 64) ? 6 : 5;
+  static constexpr uint32_t MASK = (1u << KB) - 1u;
+  static constexpr int kCapF = (1 << (16 - KB)) - 1;
+  static constexpr int kCapI = (1 << (15 - KB)) - 1;
+  static constexpr int kTileWords = BS * BS / 2;
+  static_assert((1 << KB) == BS && 2 * (kCapI << KB) + BS <= (1 << 16), "16-bit keys");
+};
+// What a panel tile publishes beside its snapshot: the bound of its finite
+// entries, whether an entry is INF, and whether the snapshot is of 16-bit keys.
+constexpr int kBndInf = 1 << 30, kBndH = 1 << 29;
+__host__ __device__ constexpr int bnd_value(int b) { return b & (kBndH - 1); }
+// Clamp of the 16-bit keys of two tiles with these bounds; 0 when they cannot
+// hold their sums (or a snapshot is of another kind).
+template <int BS>
+__device__ __forceinline__ int h_clamp(int ba, int bb) {
+  const int sum = bnd_value(ba) + bnd_value(bb);
+  const int cap = ((ba | bb) & kBndInf) ? KeysH<BS>::kCapI : KeysH<BS>::kCapF;
+  return (ba & bb & kBndH) && sum < cap ? cap : 0;
+}
+// Whether a panel tile relaxed over 32-bit keys or values publishes 16-bit
+// keys: below half the clamp, so that most of its partners' sums fit.
+template <int BS>
+__device__ __forceinline__ bool h_tile_ok(int bnd) {
+  return 2 * bnd_value(bnd) < ((bnd & kBndInf) ? KeysH<BS>::kCapI : KeysH<BS>::kCapF);
+}
 
 // Element types: int32 and fp32 (the relaxation of the hot path), int64 and
 // fp64 (the paper's double-precision runs, Sec. 4).  kInt: sums are exact, so
@@ -379,6 +443,9 @@ struct Args {
   T* rowR;              // raw
   int32_t* rowP;        // [2][tiles][BS*BS] predecessors of the row panel tiles
   int32_t* rowB;
+  // 16-bit key snapshots of the panel tiles (int32; KeysH, put_h): [2][tiles][BS*BS/2]
+  uint32_t* colH;
+  uint32_t* rowH;
   // 2-D tensor map of D (CUtensorMap, BS x BS boxes) for the persistent
   // driver's tile loads; null: the tile is copied row by row
   const void* tmapD;
@@ -388,6 +455,21 @@ struct Args {
   int trace_cap;
   int trace_stride;
 };
+
+// Snapshot pointers of a workspace.  An int32 solve records via codes and
+// keeps no row-panel predecessors, so its 16-bit key snapshots (2 bytes per
+// entry, two panels) fill exactly that array.
+template <typename T, class Ws>
+void set_snapshots(Args<T>& a, const Ws& ws) {
+  a.slot_tiles = ws.slot_tiles;
+  a.piv = reinterpret_cast<T*>(ws.piv); a.pivP = ws.pivP;
+  a.colK = ws.colK; a.colR = reinterpret_cast<T*>(ws.colR); a.colB = ws.colB;
+  a.rowK = ws.rowK; a.rowR = reinterpret_cast<T*>(ws.rowR); a.rowP = ws.rowP; a.rowB = ws.rowB;
+  if constexpr (Num<T>::kPacked) {
+    a.colH = reinterpret_cast<uint32_t*>(ws.rowP);
+    a.rowH = a.colH + (size_t)ws.R * ws.BS * ws.BS;  // 2 slots x R tiles x BS^2 / 2 words
+  }
+}
 
 // -------------------------------------------------------- shared memory ----
 
@@ -404,7 +486,7 @@ struct CtaScratch {
   uint64_t bar;        // mbarrier of the operand bulk copies
   int task;            // claimed task index
   int flag;            // broadcast of a thread-0 decision
-  int red[2][8];       // per-warp partial maxima
+  int red[4][8];       // per-warp partial maxima
 };
 
 // -------------------------------------------------------- tile helpers ----
@@ -545,21 +627,31 @@ __device__ __forceinline__ int32_t resolve_pred(int32_t p, const int32_t* P, int
   return p;
 }
 
-// CTA-wide maximum of two ints (every thread gets the result).
-__device__ __forceinline__ void block_max2(int& a, int& b, CtaScratch* cs) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a = max(a, __shfl_xor_sync(0xffffffffu, a, o));
-    b = max(b, __shfl_xor_sync(0xffffffffu, b, o));
-  }
+// CTA-wide maxima of N ints (every thread gets the results).
+template <int N>
+__device__ __forceinline__ void block_max(int (&v)[N], CtaScratch* cs) {
+  static_assert(N <= 4, "CtaScratch::red");
   const int w = threadIdx.x >> 5;
-  bar_compute();
-  if ((threadIdx.x & 31) == 0) { cs->red[0][w] = a; cs->red[1][w] = b; }
-  bar_compute();
-  a = cs->red[0][0];
-  b = cs->red[1][0];
 #pragma unroll
-  for (int k = 1; k < kThreads / 32; ++k) { a = max(a, cs->red[0][k]); b = max(b, cs->red[1][k]); }
+  for (int i = 0; i < N; ++i) v[i] = __reduce_max_sync(0xffffffffu, v[i]);
+  bar_compute();
+  if ((threadIdx.x & 31) == 0) {
+#pragma unroll
+    for (int i = 0; i < N; ++i) cs->red[i][w] = v[i];
+  }
+  bar_compute();
+#pragma unroll
+  for (int i = 0; i < N; ++i) {
+    v[i] = cs->red[i][0];
+#pragma unroll
+    for (int k = 1; k < kThreads / 32; ++k) v[i] = max(v[i], cs->red[i][k]);
+  }
+}
+__device__ __forceinline__ void block_max2(int& a, int& b, CtaScratch* cs) {
+  int v[2] = {a, b};
+  block_max(v, cs);
+  a = v[0];
+  b = v[1];
 }
 
 // ---------------------------------------------------------- min-plus cores ----
@@ -593,6 +685,102 @@ __device__ __forceinline__ void core_packed(const uint32_t* __restrict__ As,
 #pragma unroll
       for (int nn = 0; nn < TM; ++nn) acc[m][nn] = __viaddmin_u32(a[m], b[nn], acc[m][nn]);
   }
+}
+
+// Layout of a 16-bit snapshot (KeysH): 16-byte units of four words (eight
+// steps) of one operand row; the unit w4 of the row in micro-tile register m
+// of thread row t starts at word ((w4 * TM + m) * 16 + t) * 4, so that the
+// lanes of a warp read consecutive units.
+template <int BS>
+__device__ __forceinline__ int h_unit(int w4, int m, int t) {
+  return ((w4 * Geo<BS>::TM + m) * 16 + t) * 4;
+}
+
+// Step (0 .. BS-1) of half `half` of operand word kw (0 .. BS/2 - 1).
+template <int BS>
+__device__ __forceinline__ int kk_of(int kw, int half) {
+  constexpr int NW = KeysH<BS>::kNW;
+  return Geo<BS>::idx(kw / NW, kw % NW + NW * half);
+}
+
+// Write a micro-tile of 16-bit values as a snapshot.  val(k, r): the value of
+// this thread's register k along the inner dimension (thread index tk) and
+// register r along the operand's rows (thread index tr).
+template <int BS, bool kCode, class F>
+__device__ __forceinline__ void put_h(uint32_t* H, int tk, int tr, F&& val) {
+  constexpr int TM = Geo<BS>::TM, NW = KeysH<BS>::kNW;
+  auto word = [&](int e, int r) -> uint32_t {
+    const uint32_t kk = kCode ? (uint32_t)kk_of<BS>(tk * NW + e, 0) |
+                                    ((uint32_t)kk_of<BS>(tk * NW + e, 1) << 16)
+                              : 0u;
+    return (val(e, r) | (val(e + NW, r) << 16)) + kk;
+  };
+#pragma unroll
+  for (int r = 0; r < TM; ++r) {
+    uint32_t* u = H + h_unit<BS>(tk * NW / 4, r, tr) + tk * NW % 4;
+    if constexpr (NW == 4)
+      *reinterpret_cast<uint4*>(u) = make_uint4(word(0, r), word(1, r), word(2, r), word(3, r));
+    else if constexpr (NW == 2)
+      *reinterpret_cast<uint2*>(u) = make_uint2(word(0, r), word(1, r));
+    else
+      *u = word(0, r);
+  }
+}
+
+// Relaxation over 16-bit keys: acc's halves take the minima over the low and
+// the high steps.  Two relaxations per instruction: 122 relaxations per SM
+// clock from shared memory, where the 32-bit keys of core_packed reach 63
+// (the same DPX rate of 64 lanes per SM clock for both).  Two 32-bit adds and
+// one three-input 16-bit minimum per two words measured 115.
+template <int BS>
+__device__ __forceinline__ void core_h(const uint32_t* __restrict__ As,
+                                       const uint32_t* __restrict__ Bs,
+                                       uint32_t (&acc)[Geo<BS>::TM][Geo<BS>::TM], int tx, int ty) {
+  constexpr int TM = Geo<BS>::TM;
+  // operands one unit ahead: with one warp per SM sub-partition at work
+  // nothing else hides the loads
+  constexpr int U = BS / 8;
+  uint4 b[2][TM], an;
+#pragma unroll
+  for (int nn = 0; nn < TM; ++nn)
+    b[0][nn] = *reinterpret_cast<const uint4*>(Bs + h_unit<BS>(0, nn, tx));
+  an = *reinterpret_cast<const uint4*>(As + h_unit<BS>(0, 0, ty));
+#pragma unroll 1
+  for (int w0 = 0; w0 < U; w0 += 2) {
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const int w4 = w0 + h, nx = w4 + 1 < U ? w4 + 1 : w4;
+#pragma unroll
+      for (int m = 0; m < TM; ++m) {
+        const uint4 a = an;
+        an = *reinterpret_cast<const uint4*>(
+            As + (m + 1 < TM ? h_unit<BS>(w4, m + 1, ty) : h_unit<BS>(nx, 0, ty)));
+        b[h ^ 1][m] = *reinterpret_cast<const uint4*>(Bs + h_unit<BS>(nx, m, tx));
+#pragma unroll
+        for (int nn = 0; nn < TM; ++nn) acc[m][nn] = __viaddmin_u16x2(a.x, b[h][nn].x, acc[m][nn]);
+#pragma unroll
+        for (int nn = 0; nn < TM; ++nn) acc[m][nn] = __viaddmin_u16x2(a.y, b[h][nn].y, acc[m][nn]);
+#pragma unroll
+        for (int nn = 0; nn < TM; ++nn) acc[m][nn] = __viaddmin_u16x2(a.z, b[h][nn].z, acc[m][nn]);
+#pragma unroll
+        for (int nn = 0; nn < TM; ++nn) acc[m][nn] = __viaddmin_u16x2(a.w, b[h][nn].w, acc[m][nn]);
+      }
+    }
+  }
+}
+
+// Tile thread of a warp's lane where the operands are read as 16-bit
+// snapshots: a warp covers 4 x 8 of the 16 x 16 threads, so that an operand
+// load touches four or eight consecutive units (one 128-byte wavefront).
+__device__ __forceinline__ void h_thread(int& tx, int& ty) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  tx = (lane & 7) + 8 * (warp & 1);
+  ty = (lane >> 3) + 4 * (warp >> 1);
+}
+
+// Smaller halves of two 16-bit accumulators, x's in the low half.
+__device__ __forceinline__ uint32_t h_min2(uint32_t x, uint32_t y) {
+  return __vminu2(__byte_perm(x, y, 0x5410), __byte_perm(x, y, 0x7632));
 }
 
 // 1.0f when a < b, else 0.0f, in one instruction (PTX set with a float

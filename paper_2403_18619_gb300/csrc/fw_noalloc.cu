@@ -69,13 +69,11 @@ cudaError_t run(T* D, int32_t* P, int64_t n, int64_t ld, unsigned char* base, in
   if ((e = cudaGetLastError()) != cudaSuccess) return e;
 
   Args<T> a{};
-  a.D = D; a.P = P; a.n = n; a.ld = ld; a.R = R; a.slot_tiles = ws.slot_tiles;
+  a.D = D; a.P = P; a.n = n; a.ld = ld; a.R = R;
   a.ver = ws.ver; a.done = ws.done; a.ctr = ws.ctr; a.abort_flag = ws.abort_flag; a.status = status;
   a.stage_off = ws.stage_off; a.lookahead = (int)look; a.skip_task = -1;
   a.timeout_ns = 2000000000LL; a.packed = 1;
-  a.piv = reinterpret_cast<T*>(ws.piv); a.pivP = ws.pivP;
-  a.colK = ws.colK; a.colR = reinterpret_cast<T*>(ws.colR); a.colB = ws.colB;
-  a.rowK = ws.rowK; a.rowR = reinterpret_cast<T*>(ws.rowR); a.rowP = ws.rowP; a.rowB = ws.rowB;
+  set_snapshots(a, ws);
 
   int64_t blocks = (n * n + 255) / 256;
   if (blocks > (int64_t)sms * 8) blocks = (int64_t)sms * 8;

@@ -55,13 +55,11 @@ template <typename T, int BS>
 cudaError_t launch_bs(T* D, int32_t* P, int64_t n, int64_t ld, const fwh::SolveWs& ws,
                       const fwh::LaunchCfg& cfg, cudaStream_t s) {
   Args<T> a{};
-  a.D = D; a.P = P; a.n = n; a.ld = ld; a.R = ws.R; a.slot_tiles = ws.slot_tiles;
+  a.D = D; a.P = P; a.n = n; a.ld = ld; a.R = ws.R;
   a.ver = ws.ver; a.done = ws.done; a.ctr = ws.ctr; a.abort_flag = ws.abort_flag; a.status = ws.status;
   a.stage_off = ws.stage_off; a.lookahead = (int)cfg.lookahead; a.skip_task = cfg.skip_task;
   a.timeout_ns = cfg.timeout_ns; a.packed = cfg.packed;
-  a.piv = reinterpret_cast<T*>(ws.piv); a.pivP = ws.pivP;
-  a.colK = ws.colK; a.colR = reinterpret_cast<T*>(ws.colR); a.colB = ws.colB;
-  a.rowK = ws.rowK; a.rowR = reinterpret_cast<T*>(ws.rowR); a.rowP = ws.rowP; a.rowB = ws.rowB;
+  set_snapshots(a, ws);
   a.trace = cfg.trace; a.trace_cap = (int)cfg.trace_cap; a.trace_stride = cfg.trace_stride;
   const int R = ws.R;
   const size_t smem = Smem<BS, T>::bytes();

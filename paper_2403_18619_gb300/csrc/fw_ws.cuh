@@ -19,8 +19,8 @@
 //   * The publisher sleeps on the compute warps' task-done barrier and
 //     publishes each finished tile (the GPU-scope release), so that neither the
 //     compute warps nor the producer wait on that fence.
-// mbarriers carry "full" (transaction bytes landed) and "empty" (compute warps
-// done reading) signals.
+// mbarriers carry "full" (transaction bytes landed) and "empty" (readers done)
+// signals.
 //
 // The same engine runs one graph (fw_solve) or a batch of graphs with
 // different sizes and block sizes in one launch (fw_solve_batched): a "task
@@ -34,7 +34,9 @@ namespace fwk {
 
 // 10 warps: 8 compute, 1 producer, 1 publisher.  Three of them share one SM
 // sub-partition, whose 16K registers then cap the kernel at 168 registers per
-// thread (ptxas derives this from the launch bounds).
+// thread (ptxas derives this from the launch bounds).  (Four more warps that
+// did the epilogue of a 16-bit tile while the compute warps relaxed the next
+// starved: the relaxations hold the ALU pipe, n = 16384 300 ms against 180.)
 constexpr int kWsThreads = kThreads + 64;
 constexpr int kPubDepth = 4;  // tasks handed to the compute warps but not yet published
 // Internal task type: remaining tile (r+1, r+1) of round r followed, on the
@@ -73,9 +75,12 @@ struct WsLayout {
   __host__ __device__ static constexpr size_t ring_off() { return 0; }
   __host__ __device__ static constexpr size_t d_off() { return kRing; }
   __host__ __device__ static constexpr size_t p_off() { return kRing + kTile; }
-  __host__ __device__ static constexpr size_t bytes() {
+  // scratch of expand_h (int32): a 16-bit snapshot tile
+  static constexpr size_t kScr = Num<T>::kPacked ? (size_t)LBS * LBS / 2 * 4 : 0;
+  __host__ __device__ static constexpr size_t scr_off() {
     return kRing + kTile + (ViaPred<T>::kOn ? 0 : kPTile);
   }
+  __host__ __device__ static constexpr size_t bytes() { return scr_off() + kScr; }
   // pivot and panel tasks use the buffer from offset 0 as scratch (As, Bs of
   // elements and Ps of int32)
   static_assert(bytes() >= 2 * kTile + kPTile, "scratch of pivot / panel tasks");
@@ -85,11 +90,21 @@ struct WsLayout {
 struct WsBars {
   uint64_t desc_full[2], desc_empty[2];
   uint64_t chunk_full[2], chunk_empty[2];
-  uint64_t d_full, d_empty, p_full, p_empty, task_done;
+  uint64_t d_full, d_empty, p_full, p_empty;
+  // one completion barrier per publication slot: the compute warps may finish
+  // several tasks while one publication is under way, and a parity wait only
+  // tells the latest two phases apart
+  uint64_t task_done[kPubDepth];
   uint64_t pub_full[kPubDepth], pub_empty[kPubDepth];
-  int desc[2][8];           // t, type, r, ti, tj, fast, graph, key operands
+  int desc[2][8];           // t, type, r, ti, tj, mode, graph, key operands
   int pubq[kPubDepth][6];   // t, type, r, ti, tj, graph of tasks awaiting publication
+  int pst[kPubDepth];       // what the publisher stores for the task (kPst*; ws_panel_h)
 };
+
+// A 16-bit panel task leaves its results in shared memory and the publisher
+// stores them (store_panel): the ring stage of the live tile (the other one
+// holds the 16-bit snapshot), and whether the tile is whole and stored so.
+constexpr int kPstOn = 1, kPstStage = 2, kPstTile = 4;
 
 // Bounded wait on an mbarrier phase; false (and the timeout status) on expiry.
 // With poll_abort, a wait that has already lasted over a millisecond (normal
@@ -149,6 +164,9 @@ struct PipeCnt {
 
 // ------------------------------------------------------------ compute side ----
 
+// Operand forms of a remaining tile (key_operands).
+constexpr int kFormKA = 1, kFormKB = 2, kFormHA = 4, kFormHB = 8, kFormInfA = 16, kFormInfB = 32;
+
 // In-place decode of `count` packed keys (int32 path) back to values, for a
 // remaining tile relaxed with compare and select whose panel wrote its key
 // snapshot only (exact: every finite value was below CAP).  Compute warps
@@ -170,17 +188,59 @@ __device__ __forceinline__ void decode_keys(uint32_t* buf, int count) {
   }
 }
 
-// Operands of a compare-and-select remaining tile that arrive as keys: decode
-// them in the ring stage (bit 0: A, bit 1: B; every warp has waited for the
-// stage to fill, so no warp still reads its previous contents) and
-// synchronise the compute warps.
+// Expansion of a 16-bit snapshot tile at buf, in place, to the chunk of CK
+// steps from step ch * CK: 32-bit keys (with the code of the step for an A
+// operand) or values.  The tile goes through the scratch first, so that no
+// word is overwritten before it is read.
+template <int BS, int CK>
+__device__ __noinline__ void expand_h(uint32_t* buf, uint32_t* scr, int ch, bool keys, bool is_a,
+                                      bool has_inf) {
+  using H = KeysH<BS>;
+  using K = Keys<BS>;
+  using Gm = Geo<BS>;
+  constexpr int TM = Gm::TM;
+  bar_compute();  // (the scratch is free)
+#pragma unroll
+  for (int i = threadIdx.x * 4; i < H::kTileWords; i += kThreads * 4)
+    *reinterpret_cast<uint4*>(scr + i) = *reinterpret_cast<const uint4*>(buf + i);
+  bar_compute();
+#pragma unroll 4
+  for (int i = threadIdx.x; i < H::kTileWords; i += kThreads) {
+    const uint32_t w = scr[i];
+    const int row = Gm::idx((i >> 2) & 15, (i >> 6) % TM), kw = (i >> 6) / TM * 4 + (i & 3);
+    auto put = [&](int h) {
+      const int kk = kk_of<BS>(kw, h);
+      const int d = (int)((w >> (16 * h)) & 0xffffu) >> H::KB;
+      const bool inf = has_inf && d == H::kCapI;
+      buf[(kk - ch * CK) * BS + row] =
+          keys ? ((uint32_t)(inf ? K::CAP : d) << K::KB) + (is_a ? (uint32_t)kk + 1u : 0u)
+               : (uint32_t)(inf ? Num<int32_t>::inf() : d);
+    };
+    if constexpr (CK == BS) {
+      put(0);
+      put(1);
+    } else {
+      static_assert(CK == BS || (BS == 128 && CK == 64), "a half of the words per chunk");
+      put(ch);
+    }
+  }
+}
+
+// Operands of a remaining tile that arrive in another form than its core reads
+// (key_operands): 32-bit keys decoded to values, a 16-bit snapshot expanded,
+// in the ring stage (every warp has waited for the stage to fill, so no warp
+// still reads its previous contents); synchronises the compute warps.
 template <typename T, int BS, int CK>
-__device__ __forceinline__ void decode_chunk(unsigned char* stage, int dec) {
+__device__ __forceinline__ void decode_chunk(unsigned char* stage, unsigned char* scratch, int dec,
+                                             int ch, bool keys) {
   if constexpr (Num<T>::kPacked) {
-    if (!dec) return;
+    if (!(dec & (kFormKA | kFormKB | kFormHA | kFormHB))) return;
     uint32_t* As = reinterpret_cast<uint32_t*>(stage);
-    if (dec & 1) decode_keys<BS>(As, CK * BS);
-    if (dec & 2) decode_keys<BS>(As + CK * BS, CK * BS);
+    if (dec & kFormKA) decode_keys<BS>(As, CK * BS);
+    if (dec & kFormKB) decode_keys<BS>(As + CK * BS, CK * BS);
+    uint32_t* scr = reinterpret_cast<uint32_t*>(scratch);
+    if (dec & kFormHA) expand_h<BS, CK>(As, scr, ch, keys, true, dec & kFormInfA);
+    if (dec & kFormHB) expand_h<BS, CK>(As + CK * BS, scr, ch, keys, false, dec & kFormInfB);
     fence_proxy_async_shared();  // generic writes before the stage's next TMA fill
     bar_compute();
   }
@@ -233,7 +293,7 @@ __device__ __noinline__ bool ws_minplus_dist(TileCtx<T> c, int ti, int tj, int d
                    c.timeout_ns))
       return false;
     if (tr) cw += clock64() - w0;
-    decode_chunk<T, BS, C::CK>(ring + st * L::kStage, dec);
+    decode_chunk<T, BS, C::CK>(ring + st * L::kStage, smem + L::scr_off(), dec, ch, false);
     const T* As = reinterpret_cast<const T*>(ring + st * L::kStage);
     const T* Bs = As + C::CK * BS;
     core_min<BS, T, C::CK>(As, Bs, acc, tx, ty);
@@ -273,13 +333,118 @@ __device__ __noinline__ bool ws_minplus_dist(TileCtx<T> c, int ti, int tj, int d
   return true;
 }
 
-// Remaining-tile task (phase 4 of round r, tile ti,tj).  Returns false if an
-// operand never arrived (the kernel then stops).
+// Turns of the two groups of compute warps (0-3 and 4-7, one warp of each per
+// SM sub-partition) in the relaxation of a 16-bit tile: one group relaxes at
+// the full rate of the ALU pipe while the other stores what its previous turn
+// improved, which is bound by latency and the load/store unit (8 K SM cycles
+// per tile, whatever the layout; both groups in step 27 K cycles per tile,
+// 19 K of them relaxation).  Named barriers 2 + g: group g may go.
+__device__ __forceinline__ void turn_wait(int g) {
+  asm volatile("bar.sync %0, 256;" ::"r"(2 + g) : "memory");
+}
+__device__ __forceinline__ void turn_pass(int g) {
+  asm volatile("bar.arrive %0, 256;" ::"r"(2 + g) : "memory");
+}
+
+// Remaining-tile task over 16-bit packed keys (int32; cap: their clamp).  The
+// accumulators hold the operands' sums only; the tile's own values are read
+// from Dbuf afterwards, so that their copy has the whole relaxation to arrive
+// and nothing converts them to keys.
 template <typename T, int BS, int LBS>
-__device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, bool fast, int dec,
+__device__ __noinline__ bool ws_minplus_h(const Args<T>& a, const fwh::Task& k, int cap,
+                                          unsigned char* smem, WsBars* wb, PipeCnt& pc,
+                                          uint64_t* tr) {
+  using Gm = Geo<BS>;
+  using H = KeysH<BS>;
+  using L = WsLayout<LBS, T>;
+  constexpr int TM = Gm::TM, G = Gm::G;
+  const int lane = threadIdx.x & 31;
+  int tx, ty;
+  h_thread(tx, ty);
+  const T* const Dbuf = reinterpret_cast<const T*>(smem + L::d_off());
+  const unsigned st = pc.chunk & 1;
+  const long long t_a = tr ? clock64() : 0;
+  if (!mbar_wait(&wb->chunk_full[st], (pc.chunk >> 1) & 1, a.status, a.abort_flag, a.timeout_ns))
+    return false;
+  const long long cw = tr ? clock64() - t_a : 0;
+  uint32_t acc[TM][TM];
+#pragma unroll
+  for (int m = 0; m < TM; ++m)
+#pragma unroll
+    for (int nn = 0; nn < TM; ++nn) acc[m][nn] = 0xffffffffu;
+  const int group = (int)threadIdx.x >> 7;
+  turn_wait(group);
+  const uint32_t* const As = reinterpret_cast<const uint32_t*>(smem + L::ring_off() + st * L::kStage);
+  core_h<BS>(As, As + H::kTileWords, acc, tx, ty);
+  turn_pass(group ^ 1);
+  __syncwarp();
+  if (lane == 0) mbar_arrive(&wb->chunk_empty[st]);
+  ++pc.chunk;
+  const long long t_b = tr ? clock64() : 0;
+  if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns)) return false;
+  if (tr) {
+    tr[7] = cyc20(clock64() - t_b) | (cyc20(cw) << 20);
+    tr[8] = (uint64_t)(t_b - t_a);
+  }
+  const int64_t ld = a.ld, row0 = (int64_t)k.ti * BS, col0 = (int64_t)k.tj * BS;
+  const int nrow = (int)(a.n - row0 < BS ? a.n - row0 : BS);
+  const int ncol = (int)(a.n - col0 < BS ? a.n - col0 : BS);
+  const bool whole = nrow == BS && ncol == BS;
+  T* const D = a.D + row0 * ld + col0;
+  int32_t* const P = a.P ? a.P + row0 * ld + col0 : nullptr;
+  const int32_t via0 = via_code((int64_t)k.r * BS);  // via_code(k) = via0 - kk
+#pragma unroll
+  for (int m = 0; m < TM; ++m) {
+    const int lr = Gm::idx(ty, m);
+    T* const Drow = D + lr * ld;
+    int32_t* const Prow = P + lr * ld;
+#pragma unroll
+    for (int g = 0; g < Gm::NG; ++g) {
+      const int lc = g * Gm::SPAN + tx * G;
+      T v[G];
+      vload_s<G>(v, Dbuf + lr * BS + lc);
+      int kk[G];
+      bool better[G], any = false;
+#pragma unroll
+      for (int e = 0; e < G; e += 2) {
+        const uint32_t mm = h_min2(acc[m][g * G + e], acc[m][g * G + e + 1]);
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int d = h ? (int)(mm >> (16 + H::KB)) : (int)((mm >> H::KB) & (H::kCapF));
+          kk[e + h] = (int)((h ? mm >> 16 : mm) & H::MASK);
+          // (sums with an INF operand are at or above the clamp)
+          better[e + h] = d < (int)v[e + h] && d < cap && lr < nrow && lc + e + h < ncol;
+          if (better[e + h]) v[e + h] = (T)d;
+          any |= better[e + h];
+        }
+      }
+      if (whole) {
+        st_if(any, Drow + lc, v);
+      } else {
+#pragma unroll
+        for (int e = 0; e < G; ++e) st_if(better[e], Drow + lc + e, v[e]);
+      }
+      if (P) {
+#pragma unroll
+        for (int e = 0; e < G; ++e) st_if(better[e], Prow + lc + e, via0 - kk[e]);
+      }
+    }
+  }
+  __syncwarp();
+  if (lane == 0) mbar_arrive(&wb->d_empty);
+  ++pc.d;
+  if (tr) tr[8] |= (uint64_t)(clock64() - t_a) << 32;
+  return true;
+}
+
+// Remaining-tile task (phase 4 of round r, tile ti,tj).  mode: 0 compare and
+// select, 1 packed 32-bit keys (16-bit keys: ws_minplus_h).  Returns false if
+// an operand never arrived (the kernel then stops).
+template <typename T, int BS, int LBS>
+__device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mode, int dec,
                                         unsigned char* smem, WsBars* wb, PipeCnt& pc,
                                         uint64_t* tr) {
-  if (!fast && !c.P) return ws_minplus_dist<T, BS, LBS>(c, ti, tj, dec, smem, wb, pc, tr);
+  if (mode == 0 && !c.P) return ws_minplus_dist<T, BS, LBS>(c, ti, tj, dec, smem, wb, pc, tr);
   using Gm = Geo<BS>;
   using K = Keys<BS>;
   using L = WsLayout<LBS, T>;
@@ -323,7 +488,7 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, bool fa
   T* Drow = c.D + row0 * c.ld + col0;
   int32_t* Prow = c.P + row0 * c.ld + col0;
   bool neg = false;
-  if (kPacked && fast) {  // (packed keys: int32 only)
+  if (kPacked && mode) {  // (packed keys: int32 only)
     uint32_t acc[TM][TM];
     int32_t omax = 0;
 #pragma unroll
@@ -341,6 +506,7 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, bool fa
                      c.timeout_ns))
         return false;
       if (tr) cw += clock64() - w0;
+      decode_chunk<T, BS, C::CK>(ring + st * L::kStage, smem + L::scr_off(), dec, ch, true);
       const uint32_t* As = reinterpret_cast<const uint32_t*>(ring + st * L::kStage);
       const uint32_t* Bs = As + C::CK * BS;
       core_packed<BS, C::CK>(As, Bs, acc, tx, ty);
@@ -421,7 +587,7 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, bool fa
                      c.timeout_ns))
         return false;
       if (tr) cw += clock64() - w0;
-      decode_chunk<T, BS, C::CK>(ring + st * L::kStage, dec);
+      decode_chunk<T, BS, C::CK>(ring + st * L::kStage, smem + L::scr_off(), dec, ch, false);
       const T* As = reinterpret_cast<const T*>(ring + st * L::kStage);
       const T* Bs = As + C::CK * BS;
       core_generic<BS, T, C::CK, false>(As, Bs, old, arg, tx, ty, ch * C::CK);
@@ -553,17 +719,21 @@ __device__ __noinline__ bool ws_panel_finish(const Args<T>& a, int r, int t, T* 
     if constexpr (kFast) return acc[m][nn] & ~K::MASK;
     else return key_of<BS>((int32_t)acc[m][nn]);
   };
-  int nb = 0;
+  int nb = 0, has_inf = 0;
 #pragma unroll
   for (int m = 0; m < TM; ++m)
 #pragma unroll
-    for (int nn = 0; nn < TM; ++nn) nb = max(nb, bound_of<BS>(value(m, nn)));
-  int dummy = 0;
-  block_max2(nb, dummy, cs);
-  // keys are exact while every finite value is below CAP; otherwise (or
-  // without packed keys) the raw snapshot is written as well
-  const bool keys = a.packed != 0;
-  const bool raw = !keys || nb >= K::CAP;
+    for (int nn = 0; nn < TM; ++nn) {
+      nb = max(nb, bound_of<BS>(value(m, nn)));
+      has_inf |= Num<T>::finite(value(m, nn)) ? 0 : kBndInf;
+    }
+  block_max2(nb, has_inf, cs);
+  // one snapshot: 16-bit keys where the bound allows them, else 32-bit keys,
+  // which are exact while every finite value is below CAP; beyond that the raw
+  // values as well, and without packed keys the raw values only
+  const bool hok = a.packed && h_tile_ok<BS>(nb | has_inf);
+  const bool keys = a.packed && !hok;
+  const bool raw = !a.packed || nb >= K::CAP;
   const int slot = r & 1;
   const size_t tile_off = ((size_t)slot * a.slot_tiles + t) * BS * BS;
   // the pointers and sizes in registers: through the reference every access
@@ -653,9 +823,156 @@ __device__ __noinline__ bool ws_panel_finish(const Args<T>& a, int r, int t, T* 
       }
     }
   }
-  if (tid == 0) *bnd = nb;
+  if (hok) {
+    // 16-bit keys: INF is the only value at or above the clamp
+    uint32_t* const snapH = (is_row ? a.rowH : a.colH) +
+                            ((size_t)slot * a.slot_tiles + t) * KeysH<BS>::kTileWords;
+    auto key16 = [&](int m, int nn) -> uint32_t {
+      const uint32_t v = (uint32_t)min((int32_t)value(m, nn), KeysH<BS>::kCapF);
+      return (has_inf ? min(v, (uint32_t)KeysH<BS>::kCapI) : v) << KeysH<BS>::KB;
+    };
+    if constexpr (is_row)
+      put_h<BS, false>(snapH, ty, tx, [&](int k, int q) { return key16(k, q); });
+    else
+      put_h<BS, true>(snapH, tx, ty, [&](int k, int q) { return key16(q, k); });
+  }
+  if (tid == 0) *bnd = nb | has_inf | (hok ? kBndH : 0);
   stamp(3);
   return true;
+}
+
+// Relaxation over 16-bit keys and results of a producer-fed panel task whose
+// operands are staged in the scratch stage (A at its start, then B); the
+// tile's own values are in Dbuf, cap is the clamp of the operands' keys.  The
+// live tile and the 16-bit snapshot are formed in the two ring stages and the
+// publisher stores them in bulk (store_panel).  The accumulators go through
+// shared memory and a short loop decodes them: decoded in registers, the
+// unrolled code of 64 entries runs once per task from a cold instruction
+// cache (8-14 K SM cycles for what the loop does in 3 K).  The results'
+// finite values are below cap, so the tile always has a 16-bit snapshot and
+// needs no other.
+template <typename T, int BS, int LBS, bool is_row>
+__device__ __forceinline__ void ws_panel_h(const Args<T>& a, int r, int t, int cap,
+                                           unsigned char* smem, WsBars* wb, CtaScratch* cs,
+                                           PipeCnt& pc, unsigned pslot) {
+  using Gm = Geo<BS>;
+  using H = KeysH<BS>;
+  using L = WsLayout<LBS, T>;
+  constexpr int TM = Gm::TM, G = Gm::G, NW = H::kNW;
+  int tx, ty;
+  h_thread(tx, ty);
+  const unsigned s0 = pc.chunk & 1, s1 = s0 ^ 1;
+  const T* const own = reinterpret_cast<const T*>(smem + L::d_off());
+  uint32_t* const tile = reinterpret_cast<uint32_t*>(smem + L::ring_off() + s0 * L::kStage);
+  uint32_t* const hst = reinterpret_cast<uint32_t*>(smem + L::ring_off() + s1 * L::kStage);
+  uint32_t acc[TM][TM];
+#pragma unroll
+  for (int m = 0; m < TM; ++m)
+#pragma unroll
+    for (int nn = 0; nn < TM; ++nn) acc[m][nn] = 0xffffffffu;
+  core_h<BS>(hst, hst + H::kTileWords, acc, tx, ty);
+  stamp(2);
+  put_tile<BS, false>(tile, acc, tx, ty);  // (the pivot it held is in the operands)
+  bar_compute();                           // every warp has left the operands
+
+  const int64_t row0 = (int64_t)(is_row ? r : t) * BS, col0 = (int64_t)(is_row ? t : r) * BS;
+  const int64_t n = a.n, ld = a.ld;
+  const int nrow = (int)(n - row0 < BS ? n - row0 : BS);
+  const int ncol = (int)(n - col0 < BS ? n - col0 : BS);
+  const bool whole = nrow == BS && ncol == BS;
+  T* const D = a.D + row0 * ld + col0;
+  int32_t* const P = a.P ? a.P + row0 * ld + col0 : nullptr;
+  const int32_t via0 = via_code((int64_t)r * BS);  // via_code(k) = via0 - kk
+  int res[2] = {0, 0};  // bound of the finite results; any INF
+  // the 16-bit snapshot words of thread row tk along the inner dimension and
+  // operand row x, and the tile's entries behind them
+#pragma unroll 1
+  for (int i = threadIdx.x; i < BS * 16; i += kThreads) {
+    const int x = is_row ? i % BS : i / 16, tk = is_row ? i / BS : i % 16;
+    uint32_t word[NW], sum[2 * NW];
+    T v[2 * NW];
+    auto at = [&](int j) {  // entry j: half j / NW of word j % NW
+      const int kk = Gm::idx(tk, j);
+      return (is_row ? kk : x) * BS + (is_row ? x : kk);
+    };
+#pragma unroll
+    for (int j = 0; j < 2 * NW; ++j) {
+      sum[j] = tile[at(j)];
+      v[j] = own[at(j)];
+    }
+#pragma unroll
+    for (int e = 0; e < NW; ++e)
+      word[e] = is_row ? 0u : (uint32_t)Gm::idx(tk, e) | ((uint32_t)Gm::idx(tk, e + NW) << 16);
+#pragma unroll
+    for (int j = 0; j < 2 * NW; ++j) {
+      const uint32_t mm = min(sum[j] & 0xffffu, sum[j] >> 16);
+      const int d = (int)(mm >> H::KB);
+      const int lr = at(j) / BS, lc = at(j) % BS;
+      const bool in = lr < nrow && lc < ncol;
+      const bool better = in && d < (int)v[j] && d < cap;
+      v[j] = better ? (T)d : in ? v[j] : Num<T>::inf();
+      const bool inf = !Num<T>::finite(v[j]);
+      tile[at(j)] = (uint32_t)v[j];
+      word[j % NW] += (uint32_t)(inf ? H::kCapI : (int)v[j]) << (H::KB + 16 * (j / NW));
+      res[0] = max(res[0], inf ? 0 : (int)v[j]);
+      res[1] |= inf ? 1 : 0;
+      if (P && better) P[lr * ld + lc] = via0 - (int32_t)(mm & H::MASK);
+    }
+    if (!whole) {
+#pragma unroll 1
+      for (int j = 0; j < 2 * NW; ++j) {
+        const int lr = at(j) / BS, lc = at(j) % BS;
+        if (lr < nrow && lc < ncol) D[lr * ld + lc] = (T)tile[lr * BS + lc];
+      }
+    }
+    const int t16 = (x % Gm::SPAN) / G, m = (x / Gm::SPAN) * G + x % G;  // x = idx(t16, m)
+    uint32_t* u = hst + h_unit<BS>(tk * NW / 4, m, t16) + tk * NW % 4;
+    if constexpr (NW == 4) *reinterpret_cast<uint4*>(u) = make_uint4(word[0], word[1], word[2], word[3]);
+    else if constexpr (NW == 2) *reinterpret_cast<uint2*>(u) = make_uint2(word[0], word[1]);
+    else *u = word[0];
+  }
+  // (the publisher releases the ring stages)
+  fence_proxy_async_shared();
+  pc.chunk += 2;
+  block_max(res, cs);
+  if ((threadIdx.x & 31) == 0) mbar_arrive(&wb->d_empty);
+  ++pc.d;
+  if (threadIdx.x == 0) {
+    ((is_row ? a.rowB : a.colB) + (size_t)(r & 1) * a.slot_tiles)[t] =
+        res[0] | (res[1] ? kBndInf : 0) | kBndH;
+    wb->pst[pslot] = kPstOn | (s0 ? kPstStage : 0) | (whole ? kPstTile : 0);
+  }
+  stamp(3);
+}
+
+// Publisher's part of a 16-bit panel task: the bulk stores of its results from
+// shared memory, the release of the ring stages once they have been read, and
+// the wait for the stores themselves (the publication follows).  Whole warp.
+template <typename T, int BS, int LBS>
+__device__ void store_panel(const Args<T>& a, const fwh::Task& k, int pst, unsigned char* smem,
+                            WsBars* wb, int lane) {
+  using L = WsLayout<LBS, T>;
+  const bool is_row = k.type == 1;
+  const unsigned s0 = (pst & kPstStage) ? 1 : 0, s1 = s0 ^ 1;
+  const size_t ht = (size_t)(k.r & 1) * a.slot_tiles + (is_row ? k.tj : k.ti);
+  const int64_t row0 = (int64_t)k.ti * BS, col0 = (int64_t)k.tj * BS;
+  const T* const tile = reinterpret_cast<const T*>(smem + L::ring_off() + s0 * L::kStage);
+  if (lane == 0) {
+    bulk_s2g((is_row ? a.rowH : a.colH) + ht * KeysH<BS>::kTileWords,
+             smem + L::ring_off() + s1 * L::kStage, (unsigned)(BS * BS * 2));
+    if ((pst & kPstTile) && a.tmapD) tma_store_2d(a.tmapD, (int)col0, (int)row0, tile);
+  }
+  if ((pst & kPstTile) && !a.tmapD)
+    for (int rr = lane; rr < BS; rr += 32)
+      bulk_s2g(a.D + (row0 + rr) * a.ld + col0, tile + rr * BS, (unsigned)(BS * sizeof(T)));
+  bulk_commit_wait_read();
+  __syncwarp();
+  if (lane == 0) {
+    mbar_arrive_n(&wb->chunk_empty[0], kThreads / 32);
+    mbar_arrive_n(&wb->chunk_empty[1], kThreads / 32);
+  }
+  bulk_wait_all();
+  __syncwarp();
 }
 
 // Panel task of round r (int32), fed by the producer like a remaining tile:
@@ -670,14 +987,16 @@ __device__ __noinline__ bool ws_panel_finish(const Args<T>& a, int r, int t, T* 
 // this one stores its results.
 template <typename T, int BS, int LBS, bool is_row>
 __device__ __noinline__ bool ws_panel(const Args<T>& a, const fwh::Task& k, unsigned char* smem,
-                                      WsBars* wb, CtaScratch* cs, PipeCnt& pc) {
+                                      WsBars* wb, CtaScratch* cs, PipeCnt& pc, unsigned slot) {
   static_assert(Num<T>::kPacked, "producer-fed panels are the int32 path");
   using Gm = Geo<BS>;
   using K = Keys<BS>;
   using L = WsLayout<LBS, T>;
   static_assert(WsChunk<BS, T>::kTile <= L::kStage, "a tile per ring stage");
   constexpr int TM = Gm::TM, G = Gm::G;
-  const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
+  int tx, ty;
+  h_thread(tx, ty);
+  if (threadIdx.x == 0) wb->pst[slot] = 0;
   const int r = k.r, t = is_row ? k.tj : k.ti;
   const int64_t row0 = (int64_t)k.ti * BS, col0 = (int64_t)k.tj * BS;
   const int nrow = (int)(a.n - row0 < BS ? a.n - row0 : BS);
@@ -712,16 +1031,40 @@ __device__ __noinline__ bool ws_panel(const Args<T>& a, const fwh::Task& k, unsi
       }
     }
   }
-  int bs_ = 0, bp_ = 0;
+  // bounds of the tile and of the pivot, and whether they have an INF
+  int bnd[4] = {0, 0, 0, 0};
 #pragma unroll
   for (int m = 0; m < TM; ++m)
 #pragma unroll
     for (int nn = 0; nn < TM; ++nn) {
-      bs_ = max(bs_, bound_of<BS>(s[m][nn]));
-      bp_ = max(bp_, bound_of<BS>(pv[m][nn]));
+      bnd[0] = max(bnd[0], bound_of<BS>(s[m][nn]));
+      bnd[1] = max(bnd[1], bound_of<BS>(pv[m][nn]));
+      bnd[2] = max(bnd[2], (int)s[m][nn]);
+      bnd[3] = max(bnd[3], (int)pv[m][nn]);
     }
-  block_max2(bs_, bp_, cs);  // (its barriers also end every read of the raw buffers)
-  const bool fast = a.packed && (bs_ + bp_ < K::CAP);
+  block_max(bnd, cs);  // (its barriers also end every read of the raw buffers)
+  const bool fast = a.packed && (bnd[0] + bnd[1] < K::CAP);
+  if (a.packed) {
+    const int inf_s = Num<T>::finite((T)bnd[2]) ? 0 : kBndInf;
+    const int inf_p = Num<T>::finite((T)bnd[3]) ? 0 : kBndInf;
+    if (const int cap = h_clamp<BS>(bnd[0] | inf_s | kBndH, bnd[1] | inf_p | kBndH)) {
+      // 16-bit operands in the scratch stage: A, then B
+      auto key16 = [&](T v) -> uint32_t { return (uint32_t)min((int)v, cap) << KeysH<BS>::KB; };
+      uint32_t* const Ah = reinterpret_cast<uint32_t*>(scratch);
+      uint32_t* const Bh = Ah + KeysH<BS>::kTileWords;
+      if constexpr (is_row) {
+        put_h<BS, true>(Ah, tx, ty, [&](int kr, int q) { return key16(pv[q][kr]); });
+        put_h<BS, false>(Bh, ty, tx, [&](int kr, int q) { return key16(s[kr][q]); });
+      } else {
+        put_h<BS, true>(Ah, tx, ty, [&](int kr, int q) { return key16(s[q][kr]); });
+        put_h<BS, false>(Bh, ty, tx, [&](int kr, int q) { return key16(pv[kr][q]); });
+      }
+      bar_compute();
+      stamp(1);
+      ws_panel_h<T, BS, LBS, is_row>(a, r, t, cap, smem, wb, cs, pc, slot);
+      return true;
+    }
+  }
 
   // operands: A (transposed) into the scratch stage, B in place (natural
   // layout: the own tile in Dbuf for a row tile, the pivot for a column
@@ -758,13 +1101,18 @@ __device__ __noinline__ bool ws_panel(const Args<T>& a, const fwh::Task& k, unsi
 
 // Any task, compute-warp side.
 template <typename T, int BS, int LBS>
-__device__ bool compute_task(const Args<T>& a, const fwh::Task& k, bool fast, int dec,
+__device__ bool compute_task(const Args<T>& a, const fwh::Task& k, int mode, int dec,
                              unsigned char* smem, WsBars* wb, CtaScratch* cs, PipeCnt& pc,
-                             uint64_t* tr) {
+                             unsigned slot, uint64_t* tr) {
   using L = WsLayout<LBS, T>;
   if (k.type == 3 || k.type == kFusedTask) {
     const TileCtx<T> ctx{a.D, a.P, a.n, a.ld, k.r, a.status, a.abort_flag, a.timeout_ns};
-    const bool ok = ws_minplus<T, BS, LBS>(ctx, k.ti, k.tj, fast, dec, smem, wb, pc, tr);
+    bool ok;
+    if (Num<T>::kPacked && mode > 1) {
+      if constexpr (Num<T>::kPacked) ok = ws_minplus_h<T, BS, LBS>(a, k, mode, smem, wb, pc, tr);
+    } else {
+      ok = ws_minplus<T, BS, LBS>(ctx, k.ti, k.tj, mode, dec, smem, wb, pc, tr);
+    }
     if (!ok || k.type == 3) return ok;
     // fused: the tile's stores precede the pivot's loads of it (same CTA),
     // and every warp has left the tile's operand buffers before the pivot
@@ -776,8 +1124,8 @@ __device__ bool compute_task(const Args<T>& a, const fwh::Task& k, bool fast, in
   }
   if constexpr (Num<T>::kPacked) {
     if (k.type != 0) {
-      const bool ok = k.type == 1 ? ws_panel<T, BS, LBS, true>(a, k, smem, wb, cs, pc)
-                                  : ws_panel<T, BS, LBS, false>(a, k, smem, wb, cs, pc);
+      const bool ok = k.type == 1 ? ws_panel<T, BS, LBS, true>(a, k, smem, wb, cs, pc, slot)
+                                  : ws_panel<T, BS, LBS, false>(a, k, smem, wb, cs, pc, slot);
       if (ok && tr) {
         const long long t0 = t_stamp[0], t_end = clock64();
         tr[7] = (uint64_t)(t_stamp[1] - t0) | ((uint64_t)(t_stamp[2] - t0) << 32);
@@ -903,14 +1251,17 @@ __device__ __forceinline__ void publish(const Args<T>& a, const fwh::Task& k) {
     red_release_add(reinterpret_cast<unsigned*>(a.done + a.R + k.r), 1u);
 }
 
-// Whether a remaining-tile task may relax packed keys (int32, bounded panels).
+// How a remaining-tile task relaxes (ws_minplus's mode): 16-bit keys when the
+// sums of its panel tiles fit (their clamp), else 32-bit keys when those fit
+// (1), else compare and select (0; other types, or packed keys off).
 template <typename T, int BS>
-__device__ __forceinline__ bool packed_ok(const Args<T>& a, const fwh::Task& k) {
-  if (!(Num<T>::kPacked && a.packed && (k.type == 3 || k.type == kFusedTask))) return false;
+__device__ __forceinline__ int minplus_mode(const Args<T>& a, const fwh::Task& k) {
+  if (!(Num<T>::kPacked && a.packed && (k.type == 3 || k.type == kFusedTask))) return 0;
   const int slot = k.r & 1;
   const int ba = __ldcg(a.colB + (size_t)slot * a.slot_tiles + k.ti);
   const int bb = __ldcg(a.rowB + (size_t)slot * a.slot_tiles + k.tj);
-  return ba + bb < Keys<BS>::CAP;
+  if (const int cap = h_clamp<BS>(ba, bb)) return cap;
+  return bnd_value(ba) + bnd_value(bb) < Keys<BS>::CAP ? 1 : 0;
 }
 
 // Copy the tile (k.ti, k.tj) of D into Dbuf (whole producer warp): one 2-D
@@ -961,44 +1312,87 @@ __device__ __forceinline__ void issue_tile_load(const Args<T>& a, const fwh::Tas
   ++pc.d;
 }
 
-// Operand forms of a compare-and-select remaining tile (int32): the panel
-// snapshots it reads as keys (bit 0: A, bit 1: B) because their panels wrote
-// the exact keys only (bound below CAP, packed keys in use).
+// Operand forms of a remaining tile that does not relax 16-bit keys (int32),
+// by the bounds of its panel tiles (ws_panel writes one snapshot): kFormH*: a
+// 16-bit snapshot, to be expanded to 32-bit keys (mode 1) or values (mode 0);
+// kFormK*: 32-bit keys to be decoded to values (mode 0).
 template <typename T, int BS>
-__device__ __forceinline__ int key_operands(const Args<T>& a, const fwh::Task& k, bool fast) {
-  if (!(Num<T>::kPacked && a.packed && (k.type == 3 || k.type == kFusedTask)) || fast) return 0;
+__device__ __forceinline__ int key_operands(const Args<T>& a, const fwh::Task& k, int mode) {
+  if (!(Num<T>::kPacked && a.packed && (k.type == 3 || k.type == kFusedTask)) || mode > 1) return 0;
   const int slot = k.r & 1;
   const int ba = __ldcg(a.colB + (size_t)slot * a.slot_tiles + k.ti);
   const int bb = __ldcg(a.rowB + (size_t)slot * a.slot_tiles + k.tj);
-  return (ba < Keys<BS>::CAP ? 1 : 0) | (bb < Keys<BS>::CAP ? 2 : 0);
+  int form = ((ba & kBndInf) ? kFormInfA : 0) | ((bb & kBndInf) ? kFormInfB : 0);
+  if (ba & kBndH) form |= kFormHA;
+  else if (mode == 0 && bnd_value(ba) < Keys<BS>::CAP) form |= kFormKA;
+  if (bb & kBndH) form |= kFormHB;
+  else if (mode == 0 && bnd_value(bb) < Keys<BS>::CAP) form |= kFormKB;
+  return form;
 }
 
 // Issue the operand copies of remaining-tile task k (whole producer warp).
 template <typename T, int BS, int LBS>
-__device__ void issue_operands(const Args<T>& a, const fwh::Task& k, bool fast, int dec,
+__device__ void issue_operands(const Args<T>& a, const fwh::Task& k, int mode, int dec,
                                unsigned char* smem, WsBars* wb, PipeCnt& pc, int lane) {
   using L = WsLayout<LBS, T>;
   using C = WsChunk<BS, T>;
   fence_proxy_async();  // global data published by other CTAs, read by TMA below
   const int slot = k.r & 1;
-  issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
-  // operand chunks
   const size_t toffA = ((size_t)slot * a.slot_tiles + k.ti) * BS * BS;
   const size_t toffB = ((size_t)slot * a.slot_tiles + k.tj) * BS * BS;
-  const unsigned char* srcA = (fast || (dec & 1)) ? (const unsigned char*)(a.colK + toffA)
-                                                 : (const unsigned char*)(a.colR + toffA);
-  const unsigned char* srcB = (fast || (dec & 2)) ? (const unsigned char*)(a.rowK + toffB)
-                                                 : (const unsigned char*)(a.rowR + toffB);
+  if (mode > 1) {
+    // 16-bit keys: both whole operand tiles in one stage; the tile itself is
+    // needed after the relaxation only (its buffer may still be in use)
+    static_assert(!Num<T>::kPacked || (size_t)BS * BS * 4 <= L::kStage, "two 16-bit tiles per stage");
+    constexpr unsigned bytes = BS * BS * 2;
+    if (lane == 0) {
+      const unsigned st = pc.chunk & 1;
+      if (!pc.stop && mbar_wait(&wb->chunk_empty[st], ((pc.chunk >> 1) & 1) ^ 1, a.status,
+                                a.abort_flag, a.timeout_ns)) {
+        mbar_expect_tx(&wb->chunk_full[st], 2 * bytes);
+        unsigned char* dst = smem + L::ring_off() + st * L::kStage;
+        bulk_g2s(dst, a.colH + toffA / 2, bytes, &wb->chunk_full[st]);
+        bulk_g2s(dst + bytes, a.rowH + toffB / 2, bytes, &wb->chunk_full[st]);
+        pc.chunk_armed[st] = pc.chunk + 1;
+      } else {
+        pc.stop = true;
+      }
+    }
+    ++pc.chunk;
+    issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
+    return;
+  }
+  issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
+  // operand chunks
+  const unsigned char* srcA = (mode || (dec & kFormKA)) ? (const unsigned char*)(a.colK + toffA)
+                                                       : (const unsigned char*)(a.colR + toffA);
+  const unsigned char* srcB = (mode || (dec & kFormKB)) ? (const unsigned char*)(a.rowK + toffB)
+                                                       : (const unsigned char*)(a.rowR + toffB);
+  // (a 16-bit tile comes whole with every chunk, which expands its part of it)
+  unsigned bytesA = (unsigned)C::kChunkBytes, bytesB = bytesA;
+  size_t stepA = C::kChunkBytes, stepB = stepA;
+  if constexpr (Num<T>::kPacked) {
+    static_assert((size_t)BS * BS * 2 <= C::kChunkBytes, "a 16-bit tile per operand chunk");
+    if (dec & kFormHA) {
+      srcA = (const unsigned char*)(a.colH + toffA / 2);
+      bytesA = BS * BS * 2;
+      stepA = 0;
+    }
+    if (dec & kFormHB) {
+      srcB = (const unsigned char*)(a.rowH + toffB / 2);
+      bytesB = BS * BS * 2;
+      stepB = 0;
+    }
+  }
   for (int c = 0; c < C::NC; ++c) {
     if (lane == 0) {
       const unsigned st = pc.chunk & 1;
       if (!pc.stop && mbar_wait(&wb->chunk_empty[st], ((pc.chunk >> 1) & 1) ^ 1, a.status,
                                 a.abort_flag, a.timeout_ns)) {
-        mbar_expect_tx(&wb->chunk_full[st], 2 * (unsigned)C::kChunkBytes);
+        mbar_expect_tx(&wb->chunk_full[st], bytesA + bytesB);
         unsigned char* dst = smem + L::ring_off() + st * L::kStage;
-        bulk_g2s(dst, srcA + c * C::kChunkBytes, (unsigned)C::kChunkBytes, &wb->chunk_full[st]);
-        bulk_g2s(dst + C::kChunkBytes, srcB + c * C::kChunkBytes, (unsigned)C::kChunkBytes,
-                 &wb->chunk_full[st]);
+        bulk_g2s(dst, srcA + c * stepA, bytesA, &wb->chunk_full[st]);
+        bulk_g2s(dst + C::kChunkBytes, srcB + c * stepB, bytesB, &wb->chunk_full[st]);
         pc.chunk_armed[st] = pc.chunk + 1;
       } else {
         pc.stop = true;
@@ -1106,10 +1500,11 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
     mbar_init(&wb.d_empty, kThreads / 32);
     mbar_init(&wb.p_full, 1);
     mbar_init(&wb.p_empty, kThreads / 32);
-    mbar_init(&wb.task_done, kThreads / 32);
     for (int i = 0; i < kPubDepth; ++i) {
       mbar_init(&wb.pub_full[i], 1);
       mbar_init(&wb.pub_empty[i], 1);
+      mbar_init(&wb.task_done[i], kThreads / 32);
+      wb.pst[i] = 0;
     }
     fence_mbar_init();
   }
@@ -1117,21 +1512,37 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
 
   if (warp == kThreads / 32 + 1) {
     // ----------------------------------------------------------- publisher
-    if (lane == 0) {
-      for (unsigned i = 0;; ++i) {
-        const unsigned q = i % kPubDepth, ph = (i / kPubDepth) & 1;
-        if (!mbar_wait(&wb.pub_full[q], ph, src.status, src.abort_flag, src.timeout_ns)) break;
-        const int t = wb.pubq[q][0];
-        const fwh::Task k{wb.pubq[q][1], wb.pubq[q][2], wb.pubq[q][3], wb.pubq[q][4]};
-        const int g = wb.pubq[q][5];
-        if (t < 0) break;
-        // tasks finish in hand-off order: the i-th completion is this task
-        if (!mbar_wait(&wb.task_done, i & 1, src.status, src.abort_flag, src.timeout_ns)) break;
+    for (unsigned i = 0;; ++i) {
+      const unsigned q = i % kPubDepth, ph = (i / kPubDepth) & 1;
+      bool ok = true;
+      if (lane == 0) ok = mbar_wait(&wb.pub_full[q], ph, src.status, src.abort_flag, src.timeout_ns);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      __syncwarp();
+      if (!ok) break;
+      const int t = wb.pubq[q][0];
+      const fwh::Task k{wb.pubq[q][1], wb.pubq[q][2], wb.pubq[q][3], wb.pubq[q][4]};
+      const int g = wb.pubq[q][5];
+      if (t < 0) break;
+      // tasks finish in hand-off order: the i-th completion is this task
+      if (lane == 0) ok = mbar_wait(&wb.task_done[q], ph, src.status, src.abort_flag, src.timeout_ns);
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      __syncwarp();
+      if (!ok) break;
+      if constexpr (Num<T>::kPacked) {
+        const int pst = (k.type == 1 || k.type == 2) ? wb.pst[q] : 0;
+        if (pst & kPstOn)
+          with_bs<kFixedBS, LBS>(src.bs(g), [&](auto B) {
+            store_panel<T, decltype(B)::value, LBS>(src.args(g), k, pst, smem, &wb, lane);
+            return 0;
+          });
+      }
+      if (lane == 0) {
         if (t != src.skip_task) publish(src.args(g), k);
         if (uint64_t* tr = trace_slot(src.trace, src.trace_cap, src.trace_stride, t))
           tr[5] = globaltimer();
         mbar_arrive(&wb.pub_empty[q]);
       }
+      __syncwarp();
     }
     return;
   }
@@ -1172,16 +1583,16 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
           tr[3] = globaltimer();
         }
       }
-      bool fast = false;
+      int mode = 0;
       int dec = 0;
       int bs = 0;
       if (t >= 0) {
         bs = src.bs(g);
-        fast = with_bs<kFixedBS, LBS>(bs, [&](auto B) {
-          return packed_ok<T, decltype(B)::value>(src.args(g), k);
+        mode = with_bs<kFixedBS, LBS>(bs, [&](auto B) {
+          return minplus_mode<T, decltype(B)::value>(src.args(g), k);
         });
         dec = with_bs<kFixedBS, LBS>(bs, [&](auto B) {
-          return key_operands<T, decltype(B)::value>(src.args(g), k, fast);
+          return key_operands<T, decltype(B)::value>(src.args(g), k, mode);
         });
       }
       unsigned pq = 0;
@@ -1205,7 +1616,7 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
         wb.desc[ds][2] = k.r;
         wb.desc[ds][3] = k.ti;
         wb.desc[ds][4] = k.tj;
-        wb.desc[ds][5] = fast ? 1 : 0;
+        wb.desc[ds][5] = mode;
         wb.desc[ds][6] = g;
         wb.desc[ds][7] = dec;
         mbar_arrive(&wb.desc_full[ds]);
@@ -1215,7 +1626,7 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
       if (t < 0) break;
       if (k.type == 3 || k.type == kFusedTask) {
         with_bs<kFixedBS, LBS>(bs, [&](auto B) {
-          issue_operands<T, decltype(B)::value, LBS>(src.args(g), k, fast, dec, smem, &wb, pc,
+          issue_operands<T, decltype(B)::value, LBS>(src.args(g), k, mode, dec, smem, &wb, pc,
                                                      lane);
           return 0;
         });
@@ -1266,6 +1677,7 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
   }
 
   // -------------------------------------------------------------- compute
+  if (warp >= kThreads / 64) turn_pass(0);  // group 0 has the first turn
   unsigned idesc = 0;
   PipeCnt pc;
   for (;;) {
@@ -1275,7 +1687,7 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
       break;
     const int t = wb.desc[ds][0];
     const fwh::Task k{wb.desc[ds][1], wb.desc[ds][2], wb.desc[ds][3], wb.desc[ds][4]};
-    const bool fast = wb.desc[ds][5] != 0;
+    const int mode = wb.desc[ds][5];
     const int g = wb.desc[ds][6];
     const int dec = wb.desc[ds][7];
     __syncwarp();
@@ -1285,13 +1697,13 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
     uint64_t* tr = tid == 0 ? trace_slot(src.trace, src.trace_cap, src.trace_stride, t) : nullptr;
     if (tr) tr[6] = globaltimer();
     const bool ok = with_bs<kFixedBS, LBS>(src.bs(g), [&](auto B) {
-      return compute_task<T, decltype(B)::value, LBS>(src.args(g), k, fast, dec, smem, &wb, &cs,
-                                                      pc, tr);
+      return compute_task<T, decltype(B)::value, LBS>(src.args(g), k, mode, dec, smem, &wb, &cs,
+                                                      pc, (idesc - 1) % kPubDepth, tr);
     });
     if (tr) tr[9] = globaltimer();
     if (!ok) break;
     __syncwarp();
-    if (lane == 0) mbar_arrive(&wb.task_done);
+    if (lane == 0) mbar_arrive(&wb.task_done[(idesc - 1) % kPubDepth]);
   }
 }
 
