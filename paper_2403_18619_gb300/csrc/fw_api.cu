@@ -115,10 +115,11 @@ int kernel_setup(const void* fn, size_t smem, int threads) {
 
 size_t solve_ws_bytes(int R, int BS, int esize) {
   const size_t t = (size_t)BS * BS;
-  const size_t keys = esize == 4 ? 2 : 0;  // packed-key snapshots (32-bit elements only)
+  const size_t keys = esize == 4 ? 2 : 1;  // packed-key (64-bit elements: 16-bit) snapshots
   size_t b = 0;
   b += up(((size_t)R * R + 2 * (size_t)R) * 4 + 4 * 4 + 4);  // ver + done + ctr + abort
   b += up((size_t)(R + 2) * 4);              // stage offsets
+  b += up((size_t)R * 4);                    // exponents of the 16-bit bounds
   b += up(2 * t * esize) + up(2 * t * 4);    // piv, pivP
   b += up(2 * (size_t)R * t * 4) * keys;     // colK, rowK
   b += up(2 * (size_t)R * t * esize) * 2;    // colR, rowR
@@ -138,10 +139,11 @@ SolveWs carve_solve_ws(void* base, int R, int BS, int esize) {
   w.flags_bytes = ((size_t)R * R + 2 * (size_t)R) * 4 + 4 * 4 + 4;
   p += up(w.flags_bytes);
   w.stage_off = reinterpret_cast<unsigned*>(p);  p += up((size_t)(R + 2) * 4);
+  w.qexp = reinterpret_cast<int*>(p);            p += up((size_t)R * 4);
   w.piv = p;                                     p += up(2 * t * esize);
   w.pivP = reinterpret_cast<int32_t*>(p);        p += up(2 * t * 4);
+  w.colK = reinterpret_cast<uint32_t*>(p);       p += up(2 * (size_t)R * t * 4);
   if (esize == 4) {
-    w.colK = reinterpret_cast<uint32_t*>(p);     p += up(2 * (size_t)R * t * 4);
     w.rowK = reinterpret_cast<uint32_t*>(p);     p += up(2 * (size_t)R * t * 4);
   }
   w.colR = p;                                    p += up(2 * (size_t)R * t * esize);

@@ -345,6 +345,87 @@ __device__ __forceinline__ T vmin(T a, T b) {
   else return relax_lt<T>(a, b) ? a : b;
 }
 
+// ----------------------------------------------------- 16-bit lower bounds ----
+
+// q = floor(v * 2^e) of the filtered min-plus (fw_filter.cuh): 0 .. kQMax, a
+// larger finite value kQMax, a negative one 0, INF kQInf.
+constexpr unsigned kQMax = 8191, kQInf = 16383;
+constexpr int kNoLead = -5000;  // lead() of zero, INF and negative values
+
+// Scale of a round: 2^e and 2^-e (floating types), or the right shift -e.
+struct QScale {
+  float up, dn;
+  int sh;
+};
+__device__ __forceinline__ QScale q_scale(int e) {
+  return QScale{__int_as_float((127 + e) << 23), __int_as_float((127 - e) << 23), -e};
+}
+
+// Lower bounds (q_of), the candidate test (may_improve: false only if
+// F * 2^-e >= v) and the position of a positive finite value's leading bit.
+template <typename T>
+struct Quant;
+
+__device__ __forceinline__ unsigned q_of_float(float v, float up) {
+  const float x = fminf(fmaxf(v * up, 0.0f), (float)kQMax);
+  return __float_as_uint(__fadd_rd(x, 8388608.0f)) & kQInf;  // 2^23 + floor(x)
+}
+__device__ __forceinline__ float q_to_float(unsigned F) {
+  return __uint_as_float(0x4b000000u | F) - 8388608.0f;
+}
+
+// fp64: the fp32 number below v (the leading 24 bits, by integer arithmetic:
+// conversions would share the narrow FP64 pipe).
+__device__ __forceinline__ float down_to_float(double v) {
+  const long long b = __double_as_longlong(v);
+  const int hi = (int)(b >> 32);
+  if (hi < 0x38100000) return 0.0f;                             // negative, or below 2^-126
+  if (hi >= 0x47f00000) return __int_as_float(0x7f7fffff);      // 2^128 and above
+  return __int_as_float((int)((unsigned)(hi - 0x38000000) << 3 | ((unsigned)b >> 29)));
+}
+template <>
+struct Quant<double> {
+  __device__ __forceinline__ static unsigned q_of(double v, const QScale& q) {
+    return Num<double>::finite(v) ? q_of_float(down_to_float(v), q.up) : kQInf;
+  }
+  __device__ __forceinline__ static bool may_improve(unsigned F, double v, const QScale& q) {
+    // against the fp32 number above v (INF: +inf)
+    const float lo = down_to_float(v);
+    const float hi = __int_as_float(lo == 0.0f ? 0x00800000 : __float_as_int(lo) + 1);
+    return q_to_float(F) * q.dn < hi;
+  }
+  __device__ __forceinline__ static int lead(double v) {
+    const int hi = (int)(__double_as_longlong(v) >> 32);
+    return hi > 0 && hi < 0x7ff00000 ? (hi >> 20) - 1023 : kNoLead;
+  }
+  static constexpr int kMinExp = -100, kMaxExp = 100;
+};
+
+template <>
+struct Quant<int64_t> {
+  __device__ __forceinline__ static unsigned q_of(int64_t v, const QScale& q) {
+    if (!Num<int64_t>::finite(v)) return kQInf;
+    const int64_t s = (v < 0 ? 0 : v) >> q.sh;
+    return s < (int64_t)kQMax ? (unsigned)s : kQMax;
+  }
+  __device__ __forceinline__ static bool may_improve(unsigned F, int64_t v, const QScale& q) {
+    return (int64_t)((uint64_t)F << q.sh) < v;
+  }
+  __device__ __forceinline__ static int lead(int64_t v) {
+    return v > 0 && Num<int64_t>::finite(v) ? 63 - __clzll(v) : kNoLead;
+  }
+  static constexpr int kMinExp = -60, kMaxExp = 0;
+};
+
+// The round's exponent from the leading bit of the closed pivot's largest
+// finite entry, which lands in [4096, 8192): the entries that matter, sums that
+// undercut an entry, lie below.  `prev`: the exponent to keep when the pivot has no such entry.
+template <typename T>
+__device__ __forceinline__ int q_exponent(int lead, int prev) {
+  if (lead == kNoLead) return prev;
+  return min(max(12 - lead, Quant<T>::kMinExp), Quant<T>::kMaxExp);
+}
+
 // Raw vector of NB bytes and G elements viewed as one value (8-byte elements).
 template <int NB> struct RawVec;
 template <> struct RawVec<16> { int4 a; };
@@ -444,8 +525,11 @@ struct Args {
   int32_t* rowP;        // [2][tiles][BS*BS] predecessors of the row panel tiles
   int32_t* rowB;
   // 16-bit key snapshots of the panel tiles (int32; KeysH, put_h): [2][tiles][BS*BS/2]
+  // (64-bit types: 16-bit lower bounds in the same layout, fw_filter.cuh)
   uint32_t* colH;
   uint32_t* rowH;
+  int* qexp;            // [R] exponent of each round's bounds (64-bit types; set by its pivot)
+  float* pivQ;          // fp32: [2][2][BS*BS] closed pivot in step groups (fw_quad.cuh): A, B
   // 2-D tensor map of D (CUtensorMap, BS x BS boxes) for the persistent
   // driver's tile loads; null: the tile is copied row by row
   const void* tmapD;
@@ -456,19 +540,21 @@ struct Args {
   int trace_stride;
 };
 
-// Snapshot pointers of a workspace.  An int32 solve records via codes and
-// keeps no row-panel predecessors, so its 16-bit key snapshots (2 bytes per
-// entry, two panels) fill exactly that array.
+// Snapshot pointers of a workspace.  The 16-bit snapshots (2 bytes per entry,
+// two panels) of an int32 solve fill the array of row-panel predecessors, which
+// it does not keep (via codes); the 64-bit types have an array of that size for
+// them.  fp32 keeps the closed pivot in step groups where an int32 solve has its
+// 32-bit keys (never used with a single tile, R = 1).
 template <typename T, class Ws>
 void set_snapshots(Args<T>& a, const Ws& ws) {
   a.slot_tiles = ws.slot_tiles;
   a.piv = reinterpret_cast<T*>(ws.piv); a.pivP = ws.pivP;
   a.colK = ws.colK; a.colR = reinterpret_cast<T*>(ws.colR); a.colB = ws.colB;
   a.rowK = ws.rowK; a.rowR = reinterpret_cast<T*>(ws.rowR); a.rowP = ws.rowP; a.rowB = ws.rowB;
-  if constexpr (Num<T>::kPacked) {
-    a.colH = reinterpret_cast<uint32_t*>(ws.rowP);
-    a.rowH = a.colH + (size_t)ws.R * ws.BS * ws.BS;  // 2 slots x R tiles x BS^2 / 2 words
-  }
+  a.pivQ = reinterpret_cast<float*>(ws.colK);
+  a.colH = Num<T>::kPacked ? reinterpret_cast<uint32_t*>(ws.rowP) : ws.colK;
+  a.rowH = a.colH + (size_t)ws.R * ws.BS * ws.BS;  // 2 slots x R tiles x BS^2 / 2 words
+  a.qexp = ws.qexp;
 }
 
 // -------------------------------------------------------- shared memory ----
@@ -1275,10 +1361,14 @@ __device__ __forceinline__ void closure_steps(T (&d)[Geo<BS>::TM][Geo<BS>::TM],
   }
 }
 
+template <int BS, bool kA>  // fw_quad.cuh
+__device__ __forceinline__ void put_quad(float* Q, const float (&v)[Geo<BS>::TM][Geo<BS>::TM], int tx,
+                                         int ty);
+
 // Eager pivot: compare and select per relaxation (fp32, 64-bit types, large
 // int32 entries).
 template <typename T, int BS>
-__device__ __noinline__ void pivot_eager(const Args<T>& a, int r, void* smem_raw) {
+__device__ __noinline__ void pivot_eager(const Args<T>& a, int r, void* smem_raw, CtaScratch* cs) {
   using Gm = Geo<BS>;
   constexpr int TM = Gm::TM;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
@@ -1296,6 +1386,23 @@ __device__ __noinline__ void pivot_eager(const Args<T>& a, int r, void* smem_raw
   stamp(1);
   closure_steps<T, BS>(d, p, smem_raw);
   stamp(2);
+  if constexpr (std::is_same<T, float>::value) {
+    if (a.R > 1) {
+      float* const Q = a.pivQ + (size_t)(r & 1) * 2 * BS * BS;
+      put_quad<BS, true>(Q, d, tx, ty);
+      put_quad<BS, false>(Q + BS * BS, d, tx, ty);
+    }
+  }
+  if constexpr (sizeof(T) == 8) {
+    // the exponent of the round's 16-bit bounds (fw_filter.cuh)
+    int lead[1] = {kNoLead};
+#pragma unroll
+    for (int mm = 0; mm < TM; ++mm)
+#pragma unroll
+      for (int nn = 0; nn < TM; ++nn) lead[0] = max(lead[0], Quant<T>::lead(d[mm][nn]));
+    block_max(lead, cs);
+    if (tid == 0) a.qexp[r] = q_exponent<T>(lead[0], r ? __ldcg(a.qexp + r - 1) : 0);
+  }
   stamp(3);
   pivot_store_dist<T, BS>(a, r, d, tx, ty);
   pivot_store_pred<T, BS>(a, r, p, tx, ty);
@@ -1346,7 +1453,7 @@ __device__ __noinline__ void task_pivot(const Args<T>& a, int r, void* smem_raw,
       return;
     }
   }
-  pivot_eager<T, BS>(a, r, smem_raw);
+  pivot_eager<T, BS>(a, r, smem_raw, cs);
 }
 
 // ------------------------------------------------------------- phase 2/3 ----

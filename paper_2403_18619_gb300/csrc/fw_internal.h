@@ -122,6 +122,7 @@ struct SolveWs {
   int* abort_flag = nullptr;
   int* status = nullptr;
   unsigned* stage_off = nullptr;
+  int* qexp = nullptr;  // [R] exponents of the 16-bit bounds
   void* piv = nullptr;
   int32_t* pivP = nullptr;
   uint32_t* colK = nullptr;
@@ -136,7 +137,8 @@ struct SolveWs {
 };
 
 // Bytes needed by a solve of R tiles of BS with esize-byte elements (4: int32
-// or fp32, with the packed-key snapshots; 8: int64 or fp64, without them).
+// or fp32, with the packed-key snapshots; 8: int64 or fp64, with one array of
+// that size for their 16-bit snapshots).
 size_t solve_ws_bytes(int R, int BS, int esize = 4);
 // Carve a workspace out of `base` (cudaMalloc'd, >= solve_ws_bytes).
 SolveWs carve_solve_ws(void* base, int R, int BS, int esize = 4);

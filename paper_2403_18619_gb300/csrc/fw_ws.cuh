@@ -8,13 +8,13 @@
 //     tasks into shared memory with TMA copies while the compute warps work
 //     on the previous task:
 //       - the tile's own D block (one 2-D tensor copy, or one copy per row) -> Dbuf
-//       - the A and B panel snapshots, 64 (fp32: 32) k-steps per chunk -> 2-stage ring
-//       - the predecessor tile of the B panel (fp32 epilogue)          -> Pbuf
-//     and, for int32 panel tasks, the tile and the closed pivot (ws_panel).
-//   * The compute warps relax (min-plus over the chunks) and store improved
-//     entries; pivot tasks (and the panels of the other element types) are
-//     run by them alone, using the shared buffer as scratch (the producer
-//     waits until such a task is published).  The task that finishes tile
+//       - the A and B panel snapshots -> 2-stage ring: whole 16-bit tiles (keys
+//         of int32, lower bounds of the 64-bit types), or chunks of 64 k-steps
+//         of 32-bit keys or values (int32 beyond 16 bits, fp32)
+//     and, for panel tasks, the tile and the closed pivot (ws_panel*).
+//   * The compute warps relax and store improved entries; pivot tasks are run
+//     by them alone, using the shared buffer as scratch (the producer waits
+//     until such a task is published).  The task that finishes tile
 //     (r+1, r+1) of round r runs the pivot of round r+1 right after it.
 //   * The publisher sleeps on the compute warps' task-done barrier and
 //     publishes each finished tile (the GPU-scope release), so that neither the
@@ -28,6 +28,8 @@
 #pragma once
 
 #include "fw_device.cuh"
+#include "fw_filter.cuh"
+#include "fw_quad.cuh"
 #include "fw_internal.h"
 
 namespace fwk {
@@ -47,50 +49,46 @@ constexpr int kPubDepth = 4;  // tasks handed to the compute warps but not yet p
 // next pivot).
 constexpr int kFusedTask = 4;
 
-// Operand chunks of a task with block size BS: CK k-steps of A and of B.
-// int32 streams 64-step chunks (2 per task at BS = 128: fewer ring hand-offs);
-// fp32 keeps 32-step chunks and spends the saved space on the predecessor
-// snapshot tile of its epilogue.
-// 64-bit elements stream 32-step chunks (BS is at most 64 for them).
+// Operand chunks of a task that streams 32-bit keys or values (int32 beyond 16
+// bits, fp32): CK k-steps of A and of B, 64 at most (2 per task at BS = 128: few
+// ring hand-offs).
 template <int BS, typename T>
 struct WsChunk {
-  static constexpr int kCKmax = (ViaPred<T>::kOn && sizeof(T) == 4) ? 64 : 32;
-  static constexpr int CK = BS < kCKmax ? BS : kCKmax;                    // k-steps per chunk
+  static constexpr int CK = BS < 64 ? BS : 64;                            // k-steps per chunk
   static constexpr int NC = BS / CK;                                      // chunks per task
-  static constexpr size_t kChunkBytes = (size_t)CK * BS * sizeof(T);      // one operand chunk
+  static constexpr size_t kChunkBytes = (size_t)CK * BS * 4;              // one operand chunk
   static constexpr size_t kTile = (size_t)BS * BS * sizeof(T);            // a tile of elements
-  static constexpr size_t kPTile = (size_t)BS * BS * 4;                   // a tile of int32 pred
+  static constexpr size_t kHTile = (size_t)BS * BS * 2;                   // a 16-bit tile
 };
 
 // Shared-memory layout sized for the largest block size LBS a launch runs:
-// the 2-stage operand ring, the tile's own D (Dbuf) and, for the floating
-// types, the row-panel predecessor snapshot (Pbuf); 192 KB for LBS = 128 with
-// 32-bit elements, 112 KB (fp64) or 96 KB (int64) for LBS = 64.
+// the 2-stage operand ring (a stage holds two 16-bit tiles, a tile of elements
+// or two 32-bit chunks), the tile's own D (Dbuf) and a scratch (int32: a 16-bit
+// tile for expand_h; other types: a list item per entry, of 2 bytes for fp32
+// and 4 for 64-bit elements); 224 KB for LBS = 128 with 32-bit elements, 112 KB
+// for LBS = 64 with 64-bit ones (two CTAs per SM).
 template <int LBS, typename T>
 struct WsLayout {
-  static constexpr size_t kStage = 2 * WsChunk<LBS, T>::kChunkBytes;  // A chunk + B chunk
-  static constexpr size_t kRing = 2 * kStage;
   static constexpr size_t kTile = WsChunk<LBS, T>::kTile;
-  static constexpr size_t kPTile = WsChunk<LBS, T>::kPTile;
+  static constexpr size_t kHTile = WsChunk<LBS, T>::kHTile;
+  static constexpr size_t kStage = sizeof(T) == 4 ? 2 * WsChunk<LBS, T>::kChunkBytes : kTile;
+  static constexpr size_t kRing = 2 * kStage;
+  static constexpr size_t kScr = sizeof(T) == 4 ? kHTile : (size_t)LBS * LBS * 4;
+  static constexpr size_t kScrWarp = kScr / (kThreads / 32);
   __host__ __device__ static constexpr size_t ring_off() { return 0; }
   __host__ __device__ static constexpr size_t d_off() { return kRing; }
-  __host__ __device__ static constexpr size_t p_off() { return kRing + kTile; }
-  // scratch of expand_h (int32): a 16-bit snapshot tile
-  static constexpr size_t kScr = Num<T>::kPacked ? (size_t)LBS * LBS / 2 * 4 : 0;
-  __host__ __device__ static constexpr size_t scr_off() {
-    return kRing + kTile + (ViaPred<T>::kOn ? 0 : kPTile);
-  }
+  __host__ __device__ static constexpr size_t scr_off() { return kRing + kTile; }
   __host__ __device__ static constexpr size_t bytes() { return scr_off() + kScr; }
-  // pivot and panel tasks use the buffer from offset 0 as scratch (As, Bs of
-  // elements and Ps of int32)
-  static_assert(bytes() >= 2 * kTile + kPTile, "scratch of pivot / panel tasks");
-  static_assert(bytes() <= 227 * 1024, "shared memory of one CTA");
+  static_assert(2 * kHTile <= kStage && kTile <= kStage, "a stage holds either");
+  // the int32 pivot uses the buffer from offset 0 as three tiles of scratch
+  static_assert(!Num<T>::kPacked || bytes() >= 3 * kTile, "scratch of pivot tasks");
+  static_assert(bytes() <= 226 * 1024, "shared memory of one CTA");
 };
 
 struct WsBars {
   uint64_t desc_full[2], desc_empty[2];
   uint64_t chunk_full[2], chunk_empty[2];
-  uint64_t d_full, d_empty, p_full, p_empty;
+  uint64_t d_full, d_empty;
   // one completion barrier per publication slot: the compute warps may finish
   // several tasks while one publication is under way, and a parity wait only
   // tells the latest two phases apart
@@ -157,8 +155,8 @@ struct TileCtx {
 // (The drain waits on the LAST phase of each barrier: a parity wait can only
 // tell the latest two phases apart.)
 struct PipeCnt {
-  unsigned d = 0, chunk = 0, p = 0;
-  unsigned d_armed = 0, p_armed = 0, chunk_armed[2] = {0, 0};
+  unsigned d = 0, chunk = 0;
+  unsigned d_armed = 0, chunk_armed[2] = {0, 0};
   bool stop = false;
 };
 
@@ -437,6 +435,382 @@ __device__ __noinline__ bool ws_minplus_h(const Args<T>& a, const fwh::Task& k, 
   return true;
 }
 
+// fp32: the parts of a QuadTask that follow from the tile (ti, tj).
+template <int BS>
+__device__ __forceinline__ QuadTask quad_task(const Args<float>& a, int ti, int tj) {
+  QuadTask f;
+  f.D = a.D + (int64_t)ti * BS * a.ld + (int64_t)tj * BS;
+  f.P = a.P ? a.P + (int64_t)ti * BS * a.ld + (int64_t)tj * BS : nullptr;
+  f.ld = a.ld;
+  f.diag = ti == tj;
+  f.status = a.status;
+  return f;
+}
+
+// Remaining-tile task of fp32.  With predecessors the groups of warps relax in
+// turns, each with the pipes to itself while the other finds the steps of what
+// it improved (n = 8192: 78 ms, 83 without turns); distances alone leave little
+// to do afterwards (n = 5000: 10.5 ms without turns, 11.9 with).
+template <int BS, int LBS>
+__device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task& k,
+                                          unsigned char* smem, WsBars* wb, PipeCnt& pc,
+                                          uint64_t* tr) {
+  using L = WsLayout<LBS, float>;
+  using C = WsChunk<BS, float>;
+  constexpr int TM = Geo<BS>::TM;
+  const int lane = threadIdx.x & 31;
+  int tx, ty;
+  h_thread(tx, ty);
+  const long long t_a = tr ? clock64() : 0;
+  long long cw = 0;
+  float acc[TM][TM];
+  uint32_t arg[TM][QuadArg<TM>::kWords];
+#pragma unroll
+  for (int m = 0; m < TM; ++m)
+#pragma unroll
+    for (int nn = 0; nn < TM; ++nn) {
+      acc[m][nn] = Num<float>::inf();
+      arg[m][nn / 4] = 0;
+    }
+  const int group = (int)threadIdx.x >> 7;
+  bool ok = mbar_wait(&wb->chunk_full[pc.chunk & 1], (pc.chunk >> 1) & 1, a.status, a.abort_flag,
+                      a.timeout_ns);
+  if (a.P) turn_wait(group);
+#pragma unroll 1
+  for (int ch = 0; ch < C::NC && ok; ++ch) {
+    const unsigned st = pc.chunk & 1;
+    const long long w0 = tr ? clock64() : 0;
+    ok = mbar_wait(&wb->chunk_full[st], (pc.chunk >> 1) & 1, a.status, a.abort_flag, a.timeout_ns);
+    if (!ok) break;
+    if (tr) cw += clock64() - w0;
+    const float* const As = reinterpret_cast<const float*>(smem + L::ring_off() + st * L::kStage);
+    const float* const Bs = As + C::CK * BS;
+    if (a.P) core_q<BS, C::CK / 4, true>(As, Bs, acc, arg, tx, ty, ch * (C::CK / 4));
+    else core_q<BS, C::CK / 4, false>(As, Bs, acc, arg, tx, ty, 0);
+    __syncwarp();
+    if (lane == 0) mbar_arrive(&wb->chunk_empty[st]);
+    ++pc.chunk;
+  }
+  if (a.P) turn_pass(group ^ 1);  // (also when a wait has given up: the other group must not wait for it)
+  if (!ok) return false;
+  const long long t_b = tr ? clock64() : 0;
+  if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns)) return false;
+  if (tr) {
+    tr[7] = cyc20(clock64() - t_b) | (cyc20(cw) << 20);
+    tr[8] = (uint64_t)(t_b - t_a);
+  }
+  QuadTask f = quad_task<BS>(a, k.ti, k.tj);
+  const size_t ta = (size_t)(k.r & 1) * a.slot_tiles + k.ti, tb = (size_t)(k.r & 1) * a.slot_tiles + k.tj;
+  f.A = a.colR + ta * BS * BS;
+  f.B = a.rowR + tb * BS * BS;
+  f.Psrc = a.rowP + tb * BS * BS;
+  const int64_t row0 = (int64_t)k.ti * BS, col0 = (int64_t)k.tj * BS;
+  finish_tile_q<BS, true>(f, reinterpret_cast<const float*>(smem + L::d_off()),
+                          (int)(a.n - row0 < BS ? a.n - row0 : BS),
+                          (int)(a.n - col0 < BS ? a.n - col0 : BS), acc, arg, tx, ty,
+                          reinterpret_cast<uint16_t*>(smem + L::scr_off() +
+                                                      (threadIdx.x >> 5) * L::kScrWarp));
+  __syncwarp();
+  if (lane == 0) mbar_arrive(&wb->d_empty);
+  ++pc.d;
+  if (tr) tr[8] |= (uint64_t)(clock64() - t_a) << 32;
+  return true;
+}
+
+// Panel task of fp32: Dbuf holds the tile's own values, ring stage s0 the closed
+// pivot in step groups, and stage s1 takes the own values in step groups.  The
+// improved entries go to the matrix; the tile's snapshots (step groups, a row
+// tile's predecessors) are made from it afterwards.  A row tile's predecessors
+// come from its own old ones, which wait in the snapshot's place meanwhile.
+template <int BS, int LBS, bool is_row>
+__device__ __noinline__ bool ws_panel_q(const Args<float>& a, const fwh::Task& k,
+                                        unsigned char* smem, WsBars* wb, PipeCnt& pc) {
+  using L = WsLayout<LBS, float>;
+  constexpr int TM = Geo<BS>::TM;
+  const int lane = threadIdx.x & 31;
+  int tx, ty;
+  h_thread(tx, ty);
+  const int r = k.r, t = is_row ? k.tj : k.ti;
+  const unsigned s0 = pc.chunk & 1, s1 = s0 ^ 1;
+  const float* const own = reinterpret_cast<const float*>(smem + L::d_off());
+  const float* const pivq = reinterpret_cast<const float*>(smem + L::ring_off() + s0 * L::kStage);
+  float* const ownq = reinterpret_cast<float*>(smem + L::ring_off() + s1 * L::kStage);
+  stamp(0);
+  QuadTask f = quad_task<BS>(a, k.ti, k.tj);
+  const int64_t row0 = (int64_t)k.ti * BS, col0 = (int64_t)k.tj * BS;
+  const int nrow = (int)(a.n - row0 < BS ? a.n - row0 : BS);
+  const int ncol = (int)(a.n - col0 < BS ? a.n - col0 : BS);
+  const size_t tile = (size_t)(r & 1) * a.slot_tiles + t;
+  int32_t* const snapP = a.rowP + tile * BS * BS;
+  if (is_row && f.P) {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < BS * BS; i += kThreads) {
+      const int lr = i / BS, lc = i % BS;
+      snapP[i] = lr < nrow && lc < ncol ? __ldcg(f.P + lr * f.ld + lc) : -1;
+    }
+  }
+  if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns) ||
+      !mbar_wait(&wb->chunk_full[s0], (pc.chunk >> 1) & 1, a.status, a.abort_flag,
+                 a.timeout_ns) ||
+      !mbar_wait(&wb->chunk_full[s1], ((pc.chunk + 1) >> 1) & 1, a.status, a.abort_flag,
+                 a.timeout_ns))
+    return false;
+  // unit (g, x): steps 4g .. 4g+3 of operand row x
+#pragma unroll 2
+  for (int i = threadIdx.x; i < BS * BS / 4; i += kThreads) {
+    const int x = is_row ? i % BS : i / (BS / 4), g = is_row ? i / BS : i % (BS / 4);
+    float v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int lr = is_row ? 4 * g + e : x, lc = is_row ? x : 4 * g + e;
+      v[e] = lr < nrow && lc < ncol ? own[lr * BS + lc] : Num<float>::inf();
+    }
+    *reinterpret_cast<float4*>(ownq + unit_of<BS>(x) + g * TM * 64) = make_float4(v[0], v[1], v[2], v[3]);
+  }
+  bar_compute();  // (and the old predecessors are in place)
+  stamp(1);
+  float acc[TM][TM];
+  uint32_t arg[TM][QuadArg<TM>::kWords];
+#pragma unroll
+  for (int m = 0; m < TM; ++m)
+#pragma unroll
+    for (int nn = 0; nn < TM; ++nn) {
+      acc[m][nn] = Num<float>::inf();
+      arg[m][nn / 4] = 0;
+    }
+  f.A = is_row ? pivq : ownq;
+  f.B = is_row ? ownq : pivq;
+  f.Psrc = is_row ? snapP : a.pivP + (size_t)(r & 1) * BS * BS;
+  core_q<BS, BS / 4, true>(f.A, f.B, acc, arg, tx, ty, 0);
+  finish_tile_q<BS, false>(f, own, nrow, ncol, acc, arg, tx, ty,
+                           reinterpret_cast<uint16_t*>(smem + L::scr_off() +
+                                                       (threadIdx.x >> 5) * L::kScrWarp));
+  fence_proxy_async_shared();  // generic writes before the stage's next TMA fill
+  bar_compute();  // the relaxed tile is in the matrix, the operands are free
+  stamp(2);
+  if (lane == 0) {
+    mbar_arrive(&wb->d_empty);
+    mbar_arrive(&wb->chunk_empty[0]);
+    mbar_arrive(&wb->chunk_empty[1]);
+  }
+  ++pc.d;
+  pc.chunk += 2;
+  float* const snapR = (is_row ? a.rowR : a.colR) + tile * BS * BS;
+#pragma unroll 2
+  for (int i = threadIdx.x; i < BS * BS / 4; i += kThreads) {
+    const int x = is_row ? i % BS : i / (BS / 4), g = is_row ? i / BS : i % (BS / 4);
+    float v[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const int lr = is_row ? 4 * g + e : x, lc = is_row ? x : 4 * g + e;
+      const bool in = lr < nrow && lc < ncol;
+      v[e] = in ? __ldcg(f.D + lr * f.ld + lc) : Num<float>::inf();
+      if (is_row && f.P && in) snapP[lr * BS + lc] = __ldcg(f.P + lr * f.ld + lc);
+    }
+    *reinterpret_cast<float4*>(snapR + unit_of<BS>(x) + g * TM * 64) = make_float4(v[0], v[1], v[2], v[3]);
+  }
+  stamp(3);
+  return true;
+}
+
+// The parts of a FilterTask that follow from the tile (ti, tj) of round r.
+template <typename T, int BS>
+__device__ __forceinline__ FilterTask<T> filter_task(const Args<T>& a, int r, int ti, int tj) {
+  const int64_t row0 = (int64_t)ti * BS, col0 = (int64_t)tj * BS, k0 = (int64_t)r * BS;
+  FilterTask<T> f;
+  f.D = a.D + row0 * a.ld + col0;
+  f.P = a.P ? a.P + row0 * a.ld + col0 : nullptr;
+  f.ld = a.ld;
+  f.nrow = (int)(a.n - row0 < BS ? a.n - row0 : BS);
+  f.ncol = (int)(a.n - col0 < BS ? a.n - col0 : BS);
+  f.kn = (int)(a.n - k0 < BS ? a.n - k0 : BS);
+  f.r = r;
+  f.bs = BS;
+  f.diag = ti == tj;
+  f.status = a.status;
+  f.q = q_scale(__ldcg(a.qexp + r));
+  f.Psrc = nullptr;
+  f.neg = false;
+  return f;
+}
+
+// Remaining-tile task of the 64-bit types: the 16-bit pass
+// in turns, then the exact relaxation of the entries that may improve while
+// the other group of warps has its turn.
+template <typename T, int BS, int LBS>
+__device__ __noinline__ bool ws_minplus_f(const Args<T>& a, const fwh::Task& k, unsigned char* smem,
+                                          WsBars* wb, PipeCnt& pc, uint64_t* tr) {
+  using H = KeysH<BS>;
+  using L = WsLayout<LBS, T>;
+  constexpr int TM = Geo<BS>::TM;
+  const int lane = threadIdx.x & 31;
+  int tx, ty;
+  h_thread(tx, ty);
+  const unsigned st = pc.chunk & 1;
+  const long long t_a = tr ? clock64() : 0;
+  if (!mbar_wait(&wb->chunk_full[st], (pc.chunk >> 1) & 1, a.status, a.abort_flag, a.timeout_ns))
+    return false;
+  const long long cw = tr ? clock64() - t_a : 0;
+  uint32_t acc[TM][TM];
+#pragma unroll
+  for (int m = 0; m < TM; ++m)
+#pragma unroll
+    for (int nn = 0; nn < TM; ++nn) acc[m][nn] = 0xffffffffu;
+  const int group = (int)threadIdx.x >> 7;
+  turn_wait(group);
+  const uint32_t* const As = reinterpret_cast<const uint32_t*>(smem + L::ring_off() + st * L::kStage);
+  core_h<BS>(As, As + H::kTileWords, acc, tx, ty);
+  turn_pass(group ^ 1);
+  const long long t_b = tr ? clock64() : 0;
+  if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns)) return false;
+  if (tr) {
+    tr[7] = cyc20(clock64() - t_b) | (cyc20(cw) << 20);
+    tr[8] = (uint64_t)(t_b - t_a);
+  }
+  FilterTask<T> f = filter_task<T, BS>(a, k.r, k.ti, k.tj);
+  const size_t ta = (size_t)(k.r & 1) * a.slot_tiles + k.ti, tb = (size_t)(k.r & 1) * a.slot_tiles + k.tj;
+  f.A = a.colR + ta * BS * BS;
+  f.B = a.rowR + tb * BS * BS;
+  f.old = reinterpret_cast<const T*>(smem + L::d_off());
+  f.Ah = As;
+  f.Bh = As + H::kTileWords;
+  if (!ViaPred<T>::kOn) f.Psrc = a.rowP + tb * BS * BS;
+  f.neg = __ldcg(a.colB + ta) | __ldcg(a.rowB + tb);
+  refine_tile<T, BS, true>(f, acc, tx, ty,
+                     reinterpret_cast<uint32_t*>(smem + L::scr_off() + (threadIdx.x >> 5) * L::kScrWarp));
+  __syncwarp();
+  if (lane == 0) {
+    mbar_arrive(&wb->chunk_empty[st]);
+    mbar_arrive(&wb->d_empty);
+  }
+  ++pc.chunk;
+  ++pc.d;
+  if (tr) tr[8] |= (uint64_t)(clock64() - t_a) << 32;
+  return true;
+}
+
+// 16-bit bounds of a BS x BS tile in shared memory (rows and columns at or
+// beyond nrow, ncol: INF) as an A operand (steps along the columns) or a B
+// operand (steps along the rows).  Returns 1 if an entry is negative.
+template <typename T, int BS, bool kA, class Src>
+__device__ __forceinline__ int quantize_tile(uint32_t* H, const QScale& q, Src&& src) {
+  using Gm = Geo<BS>;
+  constexpr int G = Gm::G, NW = KeysH<BS>::kNW;
+  int neg = 0;
+#pragma unroll 1
+  for (int i = threadIdx.x; i < BS * 16; i += kThreads) {
+    const int x = kA ? i / 16 : i % BS, tk = kA ? i % 16 : i / BS;
+    T v[2 * NW];
+#pragma unroll
+    for (int j = 0; j < 2 * NW; ++j) {
+      const int kk = Gm::idx(tk, j);
+      v[j] = src(kA ? x : kk, kA ? kk : x);
+    }
+    uint32_t word[NW];
+#pragma unroll
+    for (int e = 0; e < NW; ++e)
+      word[e] = Quant<T>::q_of(v[e], q) | Quant<T>::q_of(v[e + NW], q) << 16;
+#pragma unroll
+    for (int j = 0; j < 2 * NW; ++j) neg |= v[j] < T(0) ? 1 : 0;
+    const int t16 = (x % Gm::SPAN) / G, m = (x / Gm::SPAN) * G + x % G;  // x = idx(t16, m)
+    uint32_t* u = H + h_unit<BS>(tk * NW / 4, m, t16) + tk * NW % 4;
+    if constexpr (NW == 4) *reinterpret_cast<uint4*>(u) = make_uint4(word[0], word[1], word[2], word[3]);
+    else if constexpr (NW == 2) *reinterpret_cast<uint2*>(u) = make_uint2(word[0], word[1]);
+    else *u = word[0];
+  }
+  return neg;
+}
+
+// Panel task of round r of the 64-bit types: Dbuf holds the tile's own values,
+// ring stage s0 the closed pivot, and stage s1 takes the 16-bit bounds of
+// both.  Filtered like a remaining tile, with its exact operands in shared
+// memory; then the tile's snapshots (values, 16-bit bounds, a row tile's
+// predecessors) are made from the relaxed tile.  A row tile's predecessors
+// come from its own old ones, which wait in the snapshot's place meanwhile.
+template <typename T, int BS, int LBS, bool is_row>
+__device__ __noinline__ bool ws_panel_f(const Args<T>& a, const fwh::Task& k, unsigned char* smem,
+                                        WsBars* wb, CtaScratch* cs, PipeCnt& pc) {
+  using H = KeysH<BS>;
+  using L = WsLayout<LBS, T>;
+  constexpr int TM = Geo<BS>::TM;
+  const int lane = threadIdx.x & 31;
+  int tx, ty;
+  h_thread(tx, ty);
+  const int r = k.r, t = is_row ? k.tj : k.ti;
+  const unsigned s0 = pc.chunk & 1, s1 = s0 ^ 1;
+  const T* const own = reinterpret_cast<const T*>(smem + L::d_off());
+  const T* const piv = reinterpret_cast<const T*>(smem + L::ring_off() + s0 * L::kStage);
+  uint32_t* const Ah = reinterpret_cast<uint32_t*>(smem + L::ring_off() + s1 * L::kStage);
+  uint32_t* const Bh = Ah + H::kTileWords;
+  stamp(0);
+  FilterTask<T> f = filter_task<T, BS>(a, r, k.ti, k.tj);
+  const size_t tile = (size_t)(r & 1) * a.slot_tiles + t;
+  int32_t* const snapP = a.rowP + tile * BS * BS;
+  if (is_row && !ViaPred<T>::kOn && f.P) {
+#pragma unroll 4
+    for (int i = threadIdx.x; i < BS * BS; i += kThreads) {
+      const int lr = i / BS, lc = i % BS;
+      snapP[i] = lr < f.nrow && lc < f.ncol ? __ldcg(f.P + lr * f.ld + lc) : -1;
+    }
+  }
+  if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns) ||
+      !mbar_wait(&wb->chunk_full[s0], (pc.chunk >> 1) & 1, a.status, a.abort_flag,
+                 a.timeout_ns) ||
+      !mbar_wait(&wb->chunk_full[s1], ((pc.chunk + 1) >> 1) & 1, a.status, a.abort_flag,
+                 a.timeout_ns))
+    return false;
+  auto own_at = [&](int i, int j) { return i < f.nrow && j < f.ncol ? own[i * BS + j] : Num<T>::inf(); };
+  auto piv_at = [&](int i, int j) { return piv[i * BS + j]; };
+  int neg[1];
+  if constexpr (is_row)
+    neg[0] = quantize_tile<T, BS, true>(Ah, f.q, piv_at) | quantize_tile<T, BS, false>(Bh, f.q, own_at);
+  else
+    neg[0] = quantize_tile<T, BS, true>(Ah, f.q, own_at) | quantize_tile<T, BS, false>(Bh, f.q, piv_at);
+  block_max(neg, cs);
+  bar_compute();  // (and the old predecessors are in place)
+  stamp(1);
+  uint32_t acc[TM][TM];
+#pragma unroll
+  for (int m = 0; m < TM; ++m)
+#pragma unroll
+    for (int nn = 0; nn < TM; ++nn) acc[m][nn] = 0xffffffffu;
+  core_h<BS>(Ah, Bh, acc, tx, ty);
+  f.A = is_row ? piv : own;
+  f.B = is_row ? own : piv;
+  f.old = own;
+  f.Ah = Ah;
+  f.Bh = Bh;
+  if (!ViaPred<T>::kOn) f.Psrc = is_row ? snapP : a.pivP + (size_t)(r & 1) * BS * BS;
+  f.neg = neg[0] != 0;
+  refine_tile<T, BS, false>(f, acc, tx, ty,
+                     reinterpret_cast<uint32_t*>(smem + L::scr_off() + (threadIdx.x >> 5) * L::kScrWarp));
+  fence_proxy_async_shared();  // generic writes before the stage's next TMA fill
+  bar_compute();  // the relaxed tile is in the matrix, the operands are free
+  stamp(2);
+  if (lane == 0) {
+    mbar_arrive(&wb->d_empty);
+    mbar_arrive(&wb->chunk_empty[0]);
+    mbar_arrive(&wb->chunk_empty[1]);
+  }
+  ++pc.d;
+  pc.chunk += 2;
+  T* const snapR = (is_row ? a.rowR : a.colR) + tile * BS * BS;
+  uint32_t* const snapH = (is_row ? a.rowH : a.colH) + tile * H::kTileWords;
+  int32_t* const Pold = is_row && !ViaPred<T>::kOn && f.P ? snapP : nullptr;
+  auto relaxed = [&](int i, int j) {
+    const bool in = i < f.nrow && j < f.ncol;
+    const T v = in ? __ldcg(f.D + i * f.ld + j) : Num<T>::inf();
+    snapR[i * BS + j] = v;
+    if (Pold && in) Pold[i * BS + j] = __ldcg(f.P + i * f.ld + j);
+    return v;
+  };
+  neg[0] = quantize_tile<T, BS, !is_row>(snapH, f.q, relaxed);
+  block_max(neg, cs);
+  if (threadIdx.x == 0) (is_row ? a.rowB : a.colB)[tile] = neg[0];
+  stamp(3);
+  return true;
+}
+
 // Remaining-tile task (phase 4 of round r, tile ti,tj).  mode: 0 compare and
 // select, 1 packed 32-bit keys (16-bit keys: ws_minplus_h).  Returns false if
 // an operand never arrived (the kernel then stops).
@@ -453,7 +827,6 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mod
   constexpr bool kPacked = Num<T>::kPacked;
   const int tid = threadIdx.x, tx = tid & 15, ty = tid >> 4, lane = tid & 31;
   const T* Dbuf = reinterpret_cast<const T*>(smem + L::d_off());
-  const int32_t* Pbuf = reinterpret_cast<const int32_t*>(smem + L::p_off());
   unsigned char* ring = smem + L::ring_off();
   const int64_t row0 = (int64_t)ti * BS, col0 = (int64_t)tj * BS;
   const int nrow = (int)(c.n - row0 < BS ? c.n - row0 : BS);  // valid rows / columns of the tile
@@ -597,12 +970,8 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mod
     }
     argmin_finish<T>(arg);
     const long long t_c = tr ? clock64() : 0;
-    if constexpr (!ViaPred<T>::kOn) {
-      // (this branch always has predecessors)
-      if (!mbar_wait(&wb->p_full, pc.p & 1, c.status, c.abort_flag, c.timeout_ns)) return false;
-    }
     if (tr) {
-      tr[7] = cyc20(t_b - t_a) | (cyc20(cw) << 20) | (cyc20(clock64() - t_c) << 40);
+      tr[7] = cyc20(t_b - t_a) | (cyc20(cw) << 20);
       tr[8] = (uint64_t)(t_c - t_a);
     }
     const int32_t via0 = via_code((int64_t)c.r * BS - 1);
@@ -615,20 +984,13 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mod
         if (arg[m][nn] && lr < nrow && lc < ncol) {
           Drow[lr * c.ld + lc] = old[m][nn];
           Prow[lr * c.ld + lc] =
-              ViaPred<T>::kOn ? via0 - arg[m][nn] : Pbuf[(arg[m][nn] - 1) * BS + lc];
+              via0 - arg[m][nn];
           neg |= (row0 + lr == col0 + lc) && old[m][nn] < T(0);
         }
       }
     }
   }
   if (tr) tr[8] |= (uint64_t)(clock64() - t_a) << 32;  // whole task
-  if constexpr (!ViaPred<T>::kOn) {
-    if (c.P) {
-      __syncwarp();
-      if (lane == 0) mbar_arrive(&wb->p_empty);
-      ++pc.p;
-    }
-  }
   if (neg) atomicOr(c.status, kStNegCycle);
   return true;
 }
@@ -1105,13 +1467,24 @@ __device__ bool compute_task(const Args<T>& a, const fwh::Task& k, int mode, int
                              unsigned char* smem, WsBars* wb, CtaScratch* cs, PipeCnt& pc,
                              unsigned slot, uint64_t* tr) {
   using L = WsLayout<LBS, T>;
+  // pivot and panel tasks: SM cycles to operands staged | relaxed ; stored |
+  // end (pivot: loads | steps ; predecessors resolved | end)
+  auto trace_stamps = [&] {
+    if (!tr) return;
+    const long long t0 = t_stamp[0], t_end = clock64();
+    tr[7] = (uint64_t)(t_stamp[1] - t0) | ((uint64_t)(t_stamp[2] - t0) << 32);
+    tr[8] = (uint64_t)(t_stamp[3] - t0) | ((uint64_t)(t_end - t0) << 32);
+  };
   if (k.type == 3 || k.type == kFusedTask) {
-    const TileCtx<T> ctx{a.D, a.P, a.n, a.ld, k.r, a.status, a.abort_flag, a.timeout_ns};
     bool ok;
-    if (Num<T>::kPacked && mode > 1) {
-      if constexpr (Num<T>::kPacked) ok = ws_minplus_h<T, BS, LBS>(a, k, mode, smem, wb, pc, tr);
+    if constexpr (Num<T>::kPacked) {
+      const TileCtx<T> ctx{a.D, a.P, a.n, a.ld, k.r, a.status, a.abort_flag, a.timeout_ns};
+      ok = mode > 1 ? ws_minplus_h<T, BS, LBS>(a, k, mode, smem, wb, pc, tr)
+                    : ws_minplus<T, BS, LBS>(ctx, k.ti, k.tj, mode, dec, smem, wb, pc, tr);
+    } else if constexpr (sizeof(T) == 4) {
+      ok = ws_minplus_q<BS, LBS>(a, k, smem, wb, pc, tr);
     } else {
-      ok = ws_minplus<T, BS, LBS>(ctx, k.ti, k.tj, mode, dec, smem, wb, pc, tr);
+      ok = ws_minplus_f<T, BS, LBS>(a, k, smem, wb, pc, tr);
     }
     if (!ok || k.type == 3) return ok;
     // fused: the tile's stores precede the pivot's loads of it (same CTA),
@@ -1122,36 +1495,27 @@ __device__ bool compute_task(const Args<T>& a, const fwh::Task& k, int mode, int
     bar_compute();
     return true;
   }
-  if constexpr (Num<T>::kPacked) {
-    if (k.type != 0) {
-      const bool ok = k.type == 1 ? ws_panel<T, BS, LBS, true>(a, k, smem, wb, cs, pc, slot)
-                                  : ws_panel<T, BS, LBS, false>(a, k, smem, wb, cs, pc, slot);
-      if (ok && tr) {
-        const long long t0 = t_stamp[0], t_end = clock64();
-        tr[7] = (uint64_t)(t_stamp[1] - t0) | ((uint64_t)(t_stamp[2] - t0) << 32);
-        tr[8] = (uint64_t)(t_stamp[3] - t0) | ((uint64_t)(t_end - t0) << 32);
-      }
-      return ok;
-    }
+  if (k.type != 0) {
+    bool ok;
+    if constexpr (Num<T>::kPacked)
+      ok = k.type == 1 ? ws_panel<T, BS, LBS, true>(a, k, smem, wb, cs, pc, slot)
+                       : ws_panel<T, BS, LBS, false>(a, k, smem, wb, cs, pc, slot);
+    else if constexpr (sizeof(T) == 4)
+      ok = k.type == 1 ? ws_panel_q<BS, LBS, true>(a, k, smem, wb, pc)
+                       : ws_panel_q<BS, LBS, false>(a, k, smem, wb, pc);
+    else
+      ok = k.type == 1 ? ws_panel_f<T, BS, LBS, true>(a, k, smem, wb, cs, pc)
+                       : ws_panel_f<T, BS, LBS, false>(a, k, smem, wb, cs, pc);
+    if (ok) trace_stamps();
+    return ok;
   }
-  // Pivot (and, for the other types, panel) tasks overwrite the ring and Dbuf
-  // from their first instructions: every compute warp must have left the
-  // previous task (a slow warp may still be reading its last operand chunk)
-  // before any warp starts.
+  // Pivot tasks overwrite the ring and Dbuf from their first instructions:
+  // every compute warp must have left the previous task (a slow warp may still
+  // be reading its last operands) before any warp starts.
   bar_compute();
-  if (k.type == 0) {
-    task_pivot<T, BS>(a, k.r, smem + L::ring_off(), cs);
-  } else {
-    task_panel<T, BS>(a, k.r, k.type == 1 ? k.tj : k.ti, k.type == 1, smem + L::ring_off(), cs);
-  }
+  task_pivot<T, BS>(a, k.r, smem + L::ring_off(), cs);
   bar_compute();
-  if (tr) {
-    // pivot: loads | steps ; predecessors resolved | end.  panel: operands
-    // staged | relaxed ; stored | end (SM cycles from the task's start)
-    const long long t0 = t_stamp[0], t_end = clock64();
-    tr[7] = (uint64_t)(t_stamp[1] - t0) | ((uint64_t)(t_stamp[2] - t0) << 32);
-    tr[8] = (uint64_t)(t_stamp[3] - t0) | ((uint64_t)(t_end - t0) << 32);
-  }
+  trace_stamps();
   return true;
 }
 
@@ -1251,12 +1615,14 @@ __device__ __forceinline__ void publish(const Args<T>& a, const fwh::Task& k) {
     red_release_add(reinterpret_cast<unsigned*>(a.done + a.R + k.r), 1u);
 }
 
-// How a remaining-tile task relaxes (ws_minplus's mode): 16-bit keys when the
-// sums of its panel tiles fit (their clamp), else 32-bit keys when those fit
-// (1), else compare and select (0; other types, or packed keys off).
+// How a remaining-tile task relaxes: int32 over 16-bit keys when the sums of
+// its panel tiles fit (their clamp), else over 32-bit keys when those fit (1),
+// else with compare and select (0; or packed keys off).  fp32: 0, in step
+// groups; 64-bit types: 2, filtered by 16-bit bounds.
 template <typename T, int BS>
 __device__ __forceinline__ int minplus_mode(const Args<T>& a, const fwh::Task& k) {
-  if (!(Num<T>::kPacked && a.packed && (k.type == 3 || k.type == kFusedTask))) return 0;
+  if (!Num<T>::kPacked) return sizeof(T) == 8 ? 2 : 0;
+  if (!(a.packed && (k.type == 3 || k.type == kFusedTask))) return 0;
   const int slot = k.r & 1;
   const int ba = __ldcg(a.colB + (size_t)slot * a.slot_tiles + k.ti);
   const int bb = __ldcg(a.rowB + (size_t)slot * a.slot_tiles + k.tj);
@@ -1343,7 +1709,6 @@ __device__ void issue_operands(const Args<T>& a, const fwh::Task& k, int mode, i
   if (mode > 1) {
     // 16-bit keys: both whole operand tiles in one stage; the tile itself is
     // needed after the relaxation only (its buffer may still be in use)
-    static_assert(!Num<T>::kPacked || (size_t)BS * BS * 4 <= L::kStage, "two 16-bit tiles per stage");
     constexpr unsigned bytes = BS * BS * 2;
     if (lane == 0) {
       const unsigned st = pc.chunk & 1;
@@ -1362,7 +1727,8 @@ __device__ void issue_operands(const Args<T>& a, const fwh::Task& k, int mode, i
     issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
     return;
   }
-  issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
+  if constexpr (sizeof(T) == 8) return;
+  if (Num<T>::kPacked) issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
   // operand chunks
   const unsigned char* srcA = (mode || (dec & kFormKA)) ? (const unsigned char*)(a.colK + toffA)
                                                        : (const unsigned char*)(a.colR + toffA);
@@ -1400,24 +1766,13 @@ __device__ void issue_operands(const Args<T>& a, const fwh::Task& k, int mode, i
     }
     ++pc.chunk;
   }
-  // predecessor tile of the row panel snapshot (fp32; int32 records "via" codes)
-  if (!ViaPred<T>::kOn && a.P) {
-    if (lane == 0) {
-      if (!pc.stop && mbar_wait(&wb->p_empty, (pc.p & 1) ^ 1, a.status, a.abort_flag, a.timeout_ns)) {
-        mbar_expect_tx(&wb->p_full, (unsigned)C::kPTile);
-        bulk_g2s(smem + L::p_off(), a.rowP + toffB, (unsigned)C::kPTile, &wb->p_full);
-        pc.p_armed = pc.p + 1;
-      } else {
-        pc.stop = true;
-      }
-    }
-    ++pc.p;
-  }
+  // (fp32 reads the tile after the relaxation: its buffer may still be in use)
+  if (!Num<T>::kPacked) issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
 }
 
-// Issue the operands of panel task k (int32, whole producer warp): the tile
-// into Dbuf, the closed pivot of round k.r into the next ring stage, and the
-// stage after it handed over empty as the task's scratch (ws_panel).
+// Issue the operands of panel task k (whole producer warp): the tile into Dbuf,
+// the closed pivot of round k.r into the next ring stage, and the stage after
+// it handed over empty as the task's scratch (ws_panel, ws_panel_f).
 template <typename T, int BS, int LBS>
 __device__ void issue_panel_operands(const Args<T>& a, const fwh::Task& k, unsigned char* smem,
                                      WsBars* wb, PipeCnt& pc, int lane) {
@@ -1430,8 +1785,10 @@ __device__ void issue_panel_operands(const Args<T>& a, const fwh::Task& k, unsig
     if (!pc.stop && mbar_wait(&wb->chunk_empty[st], ((pc.chunk >> 1) & 1) ^ 1, a.status,
                               a.abort_flag, a.timeout_ns)) {
       mbar_expect_tx(&wb->chunk_full[st], (unsigned)C::kTile);
-      bulk_g2s(smem + L::ring_off() + st * L::kStage, a.piv + (size_t)(k.r & 1) * BS * BS,
-               (unsigned)C::kTile, &wb->chunk_full[st]);
+      const void* src = a.piv + (size_t)(k.r & 1) * BS * BS;
+      if constexpr (std::is_same<T, float>::value)  // in step groups: A of a row panel, B of a column's
+        src = a.pivQ + ((size_t)(k.r & 1) * 2 + (k.type == 1 ? 0 : 1)) * BS * BS;
+      bulk_g2s(smem + L::ring_off() + st * L::kStage, src, (unsigned)C::kTile, &wb->chunk_full[st]);
       pc.chunk_armed[st] = pc.chunk + 1;
     } else {
       pc.stop = true;
@@ -1498,8 +1855,6 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
     }
     mbar_init(&wb.d_full, 1);
     mbar_init(&wb.d_empty, kThreads / 32);
-    mbar_init(&wb.p_full, 1);
-    mbar_init(&wb.p_empty, kThreads / 32);
     for (int i = 0; i < kPubDepth; ++i) {
       mbar_init(&wb.pub_full[i], 1);
       mbar_init(&wb.pub_empty[i], 1);
@@ -1636,15 +1991,15 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
           mbar_wait(&wb.pub_empty[pq], (((ipub - 1) / kPubDepth) & 1), src.status,
                     src.abort_flag, src.timeout_ns);
         }
-      } else if (Num<T>::kPacked && k.type != 0) {
+      } else if (k.type != 0) {
         with_bs<kFixedBS, LBS>(bs, [&](auto B) {
           issue_panel_operands<T, decltype(B)::value, LBS>(src.args(g), k, smem, &wb, pc, lane);
           return 0;
         });
       } else {
         if (lane == 0) {
-          // pivot / panel tasks use the shared buffer as scratch: wait until
-          // this task has been published (its publication-queue slot frees up)
+          // a pivot task uses the shared buffer as scratch: wait until it has
+          // been published (its publication-queue slot frees up)
           mbar_wait(&wb.pub_empty[pq], (((ipub - 1) / kPubDepth) & 1), src.status,
                     src.abort_flag, src.timeout_ns);
         }
@@ -1655,8 +2010,7 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
           tr[4] = globaltimer();
         }
       }
-      if (k.type == 0 || k.type == kFusedTask || (!Num<T>::kPacked && k.type != 3))
-        fence_proxy_async();
+      if (k.type == 0 || k.type == kFusedTask) fence_proxy_async();
       __syncwarp();
     }
     // leave no bulk copy in flight: wait (bounded, whatever the abort flag
@@ -1664,9 +2018,6 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
     if (lane == 0) {
       if (pc.d_armed)
         mbar_wait(&wb.d_full, (pc.d_armed - 1) & 1, src.status, src.abort_flag, src.timeout_ns,
-                  false);
-      if (pc.p_armed)
-        mbar_wait(&wb.p_full, (pc.p_armed - 1) & 1, src.status, src.abort_flag, src.timeout_ns,
                   false);
       for (int st = 0; st < 2; ++st)
         if (pc.chunk_armed[st])
@@ -1734,8 +2085,10 @@ struct SingleSrc {
   __device__ int bs(int) const { return BS; }
 };
 
+// 64-bit types: two CTAs per SM (102 registers per thread), so that the gathers
+// of one's exact relaxations overlap the other's work.
 template <typename T, int BS>
-__global__ void __launch_bounds__(kWsThreads, 1)
+__global__ void __launch_bounds__(kWsThreads, sizeof(T) == 8 ? 2 : 1)
     k_persistent_ws(Args<T> a, const __grid_constant__ CUtensorMap tmD,
                     const __grid_constant__ CUtensorMap tmP, int use_tmap) {
   extern __shared__ __align__(128) unsigned char smem[];
