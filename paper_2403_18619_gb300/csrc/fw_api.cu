@@ -521,8 +521,9 @@ fw_status fw_queue_tasks(int32_t R, int64_t lookahead, int64_t first, int64_t co
   std::vector<unsigned> off(R + 2);
   fill_stage_offsets(R, lookahead, off.data());
   if ((int64_t)off[R + 1] != total) return FW_ERR_CUDA;
+  int stage = 0;
   for (int64_t t = 0; t < count; ++t) {
-    const Task k = decode_task(first + t, R, lookahead, off.data());
+    const Task k = decode_task(first + t, R, lookahead, off.data(), stage);
     out[4 * t + 0] = k.type;
     out[4 * t + 1] = k.r;
     out[4 * t + 2] = k.ti;

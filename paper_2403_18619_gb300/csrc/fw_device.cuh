@@ -347,18 +347,28 @@ __device__ __forceinline__ T vmin(T a, T b) {
 
 // ----------------------------------------------------- 16-bit lower bounds ----
 
+// Whether the remaining tiles and panels are filtered by 16-bit bounds
+// (fw_filter.cuh): fp64 in blocks of 64.  Its exact relaxation of a tile takes
+// 160 K SM cycles there, the filtered one 400 K in the first round, where every
+// entry improves, and 20-60 K later (n = 700: 2.86 -> 2.40 ms, n = 4096: 133 ->
+// 28 ms).  At BS = 32 (n <= 512) a tile takes 19 K cycles and the rounds are
+// bound by their chain, which filtered panels lengthen (n = 400: 0.59 -> 0.68
+// ms).  int64 relaxes a tile in 36 K cycles; filtered, n = 1000 went from 1.34 to
+// 2.13 ms and n = 3000 only from 12.9 to 11.8.
+template <typename T, int BS>
+constexpr bool kFiltered = std::is_same<T, double>::value && BS == 64;
+
 // q = floor(v * 2^e) of the filtered min-plus (fw_filter.cuh): 0 .. kQMax, a
 // larger finite value kQMax, a negative one 0, INF kQInf.
 constexpr unsigned kQMax = 8191, kQInf = 16383;
 constexpr int kNoLead = -5000;  // lead() of zero, INF and negative values
 
-// Scale of a round: 2^e and 2^-e (floating types), or the right shift -e.
+// Scale of a round: 2^e and 2^-e.
 struct QScale {
   float up, dn;
-  int sh;
 };
 __device__ __forceinline__ QScale q_scale(int e) {
-  return QScale{__int_as_float((127 + e) << 23), __int_as_float((127 - e) << 23), -e};
+  return QScale{__int_as_float((127 + e) << 23), __int_as_float((127 - e) << 23)};
 }
 
 // Lower bounds (q_of), the candidate test (may_improve: false only if
@@ -399,22 +409,6 @@ struct Quant<double> {
     return hi > 0 && hi < 0x7ff00000 ? (hi >> 20) - 1023 : kNoLead;
   }
   static constexpr int kMinExp = -100, kMaxExp = 100;
-};
-
-template <>
-struct Quant<int64_t> {
-  __device__ __forceinline__ static unsigned q_of(int64_t v, const QScale& q) {
-    if (!Num<int64_t>::finite(v)) return kQInf;
-    const int64_t s = (v < 0 ? 0 : v) >> q.sh;
-    return s < (int64_t)kQMax ? (unsigned)s : kQMax;
-  }
-  __device__ __forceinline__ static bool may_improve(unsigned F, int64_t v, const QScale& q) {
-    return (int64_t)((uint64_t)F << q.sh) < v;
-  }
-  __device__ __forceinline__ static int lead(int64_t v) {
-    return v > 0 && Num<int64_t>::finite(v) ? 63 - __clzll(v) : kNoLead;
-  }
-  static constexpr int kMinExp = -60, kMaxExp = 0;
 };
 
 // The round's exponent from the leading bit of the closed pivot's largest
@@ -528,8 +522,7 @@ struct Args {
   // (64-bit types: 16-bit lower bounds in the same layout, fw_filter.cuh)
   uint32_t* colH;
   uint32_t* rowH;
-  int* qexp;            // [R] exponent of each round's bounds (64-bit types; set by its pivot)
-  float* pivQ;          // fp32: [2][2][BS*BS] closed pivot in step groups (fw_quad.cuh): A, B
+  int* qexp;            // [R] exponent of each round's bounds (fp64; set by its pivot)
   // 2-D tensor map of D (CUtensorMap, BS x BS boxes) for the persistent
   // driver's tile loads; null: the tile is copied row by row
   const void* tmapD;
@@ -542,16 +535,14 @@ struct Args {
 
 // Snapshot pointers of a workspace.  The 16-bit snapshots (2 bytes per entry,
 // two panels) of an int32 solve fill the array of row-panel predecessors, which
-// it does not keep (via codes); the 64-bit types have an array of that size for
-// them.  fp32 keeps the closed pivot in step groups where an int32 solve has its
-// 32-bit keys (never used with a single tile, R = 1).
+// it does not keep (via codes); fp64 has an array of that size for its 16-bit
+// bounds. 
 template <typename T, class Ws>
 void set_snapshots(Args<T>& a, const Ws& ws) {
   a.slot_tiles = ws.slot_tiles;
   a.piv = reinterpret_cast<T*>(ws.piv); a.pivP = ws.pivP;
   a.colK = ws.colK; a.colR = reinterpret_cast<T*>(ws.colR); a.colB = ws.colB;
   a.rowK = ws.rowK; a.rowR = reinterpret_cast<T*>(ws.rowR); a.rowP = ws.rowP; a.rowB = ws.rowB;
-  a.pivQ = reinterpret_cast<float*>(ws.colK);
   a.colH = Num<T>::kPacked ? reinterpret_cast<uint32_t*>(ws.rowP) : ws.colK;
   a.rowH = a.colH + (size_t)ws.R * ws.BS * ws.BS;  // 2 slots x R tiles x BS^2 / 2 words
   a.qexp = ws.qexp;
@@ -681,6 +672,28 @@ __device__ __forceinline__ int bound_of(T v) {
     return Keys<BS>::CAP;
   }
 }
+
+// The same bound of many int32 values, and whether one is INF, at three
+// instructions a value: subtracting 2^29 (mod 2^32) puts INF below the negative
+// numbers and these below the finite ones, so that one DPX add-and-max keeps the
+// largest finite value.  (bound_of for each: eight; with a test for INF ten, 3 K
+// of the 13 K cycles that a panel of 128 spends outside its relaxation.)
+template <int BS>
+struct Bound32 {
+  static constexpr uint32_t kInf = 1u << 29, kNonNeg = 0u - kInf;
+  uint32_t top = 0;
+  int32_t lo = 0, hi = 0;
+  __device__ __forceinline__ void add(int32_t v) {
+    top = __viaddmax_u32((uint32_t)v, kNonNeg, top);
+    lo = min(lo, v);
+    hi = max(hi, v);
+  }
+  __device__ __forceinline__ int bound() const {
+    const int b = top >= kNonNeg ? min((int)(top + kInf), Keys<BS>::CAP) : 0;
+    return lo < 0 ? Keys<BS>::CAP : b;
+  }
+  __device__ __forceinline__ int inf() const { return hi >= (int32_t)kInf ? kBndInf : 0; }
+};
 
 // Predecessors of the int32 solver ("via" encoding).  A remaining-tile task
 // that improves (i, j) through vertex k = r*BS + kk records -(k + 2) instead of
@@ -1361,10 +1374,6 @@ __device__ __forceinline__ void closure_steps(T (&d)[Geo<BS>::TM][Geo<BS>::TM],
   }
 }
 
-template <int BS, bool kA>  // fw_quad.cuh
-__device__ __forceinline__ void put_quad(float* Q, const float (&v)[Geo<BS>::TM][Geo<BS>::TM], int tx,
-                                         int ty);
-
 // Eager pivot: compare and select per relaxation (fp32, 64-bit types, large
 // int32 entries).
 template <typename T, int BS>
@@ -1386,14 +1395,7 @@ __device__ __noinline__ void pivot_eager(const Args<T>& a, int r, void* smem_raw
   stamp(1);
   closure_steps<T, BS>(d, p, smem_raw);
   stamp(2);
-  if constexpr (std::is_same<T, float>::value) {
-    if (a.R > 1) {
-      float* const Q = a.pivQ + (size_t)(r & 1) * 2 * BS * BS;
-      put_quad<BS, true>(Q, d, tx, ty);
-      put_quad<BS, false>(Q + BS * BS, d, tx, ty);
-    }
-  }
-  if constexpr (sizeof(T) == 8) {
+  if constexpr (kFiltered<T, BS>) {
     // the exponent of the round's 16-bit bounds (fw_filter.cuh)
     int lead[1] = {kNoLead};
 #pragma unroll
@@ -1442,13 +1444,14 @@ __device__ __noinline__ void task_pivot(const Args<T>& a, int r, void* smem_raw,
 #pragma unroll
         for (int nn = 0; nn < TM; ++nn) p[mm][nn] = -1;
     }
-    int bnd = 0, dummy = 0;
+    Bound32<BS> b;
 #pragma unroll
     for (int mm = 0; mm < TM; ++mm)
 #pragma unroll
-      for (int nn = 0; nn < TM; ++nn) bnd = max(bnd, bound_of<BS>(d[mm][nn]));
-    block_max2(bnd, dummy, cs);
-    if (a.packed && (int64_t)bnd * 2 * BS < (int64_t)K::CAP) {
+      for (int nn = 0; nn < TM; ++nn) b.add((int32_t)d[mm][nn]);
+    int bnd[1] = {b.bound()};
+    block_max(bnd, cs);
+    if (a.packed && (int64_t)bnd[0] * 2 * BS < (int64_t)K::CAP) {
       pivot_packed<T, BS>(a, r, smem_raw, d, p);
       return;
     }

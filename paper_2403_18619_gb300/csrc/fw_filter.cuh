@@ -1,6 +1,6 @@
-// Filtered min-plus of the 64-bit element types, whose relaxation is expensive
-// (int64: seven instructions; fp64: the narrow FP64 pipe): a 16-bit pass finds
-// the entries that can improve, and only those are relaxed exactly.
+// Filtered min-plus for element types whose relaxation is expensive (fp64: the
+// narrow FP64 pipe): a 16-bit pass finds the entries that can improve, and only
+// those are relaxed exactly.
 //
 // Operand tiles are also kept as 13-bit lower bounds, q = floor(v * 2^e) with
 // one exponent e per round (the closed pivot's largest finite entry chooses

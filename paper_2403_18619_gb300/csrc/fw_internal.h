@@ -77,14 +77,14 @@ __host__ __device__ inline Task task_panel(int R, int r, int64_t q) {
   return (q & 1) ? Task{2, r, jj, r} : Task{1, r, r, jj};
 }
 
-// off: R+2 stage starts (off[R+1] = total = R^3).
-__host__ __device__ inline Task decode_task(int64_t t, int R, int64_t look, const unsigned* off) {
-  int lo = 0, hi = R;  // find s with off[s] <= t < off[s+1]
-  while (lo < hi) {
-    const int mid = (lo + hi + 1) >> 1;
-    if ((int64_t)off[mid] <= t) lo = mid; else hi = mid - 1;
-  }
-  const int s = lo;
+// off: R+2 stage starts (off[R+1] = total = R^3).  stage: one at or before the
+// task's (a caller's tasks only advance, so that the search is a step or none);
+// receives the task's.
+__host__ __device__ inline Task decode_task(int64_t t, int R, int64_t look, const unsigned* off,
+                                            int& stage) {
+  int s = stage;
+  while (s < R && (int64_t)off[s + 1] <= t) ++s;
+  stage = s;
   int64_t u = t - (int64_t)off[s];
   if (s == R) return task_rest(R, R - 1, u);
   if (u == 0) return Task{0, s, s, s};
@@ -103,6 +103,15 @@ __host__ __device__ inline Task decode_task(int64_t t, int R, int64_t look, cons
   if (u < nrest - g) return task_rest(R, s - 1, g + u);
   u -= nrest - g;
   return task_L(R, s, u);
+}
+
+__host__ __device__ inline Task decode_task(int64_t t, int R, int64_t look, const unsigned* off) {
+  int lo = 0, hi = R;  // find s with off[s] <= t < off[s+1]
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if ((int64_t)off[mid] <= t) lo = mid; else hi = mid - 1;
+  }
+  return decode_task(t, R, look, off, lo);
 }
 
 inline void fill_stage_offsets(int R, int64_t look, unsigned* off) {

@@ -96,26 +96,6 @@ __device__ __forceinline__ uint32_t group_of(const uint32_t (&arg)[TM][QuadArg<T
   return arg[m][nn / 4] >> (nn % 4 * 8) & 63u;
 }
 
-// A micro-tile as an operand in step groups: kA: steps along the columns,
-// operand rows are the tile's rows; else steps along the rows.
-template <int BS, bool kA>
-__device__ __forceinline__ void put_quad(float* Q, const float (&v)[Geo<BS>::TM][Geo<BS>::TM], int tx,
-                                         int ty) {
-  using Gm = Geo<BS>;
-  constexpr int TM = Gm::TM, G = Gm::G;
-  const int tk = kA ? tx : ty, tr = kA ? ty : tx;
-#pragma unroll
-  for (int g = 0; g < Gm::NG; ++g)
-#pragma unroll
-    for (int r = 0; r < TM; ++r) {
-      float t[G];
-#pragma unroll
-      for (int e = 0; e < G; ++e) t[e] = kA ? v[r][g * G + e] : v[g * G + e][r];
-      const int k0 = Gm::idx(tk, g * G);
-      vstore<G>(Q + h_unit<BS>(k0 / 4, r, tr) + k0 % 4, t);
-    }
-}
-
 // First unit of operand row x = idx(t, m).
 template <int BS>
 __device__ __forceinline__ int unit_of(int x) {
@@ -127,13 +107,20 @@ __device__ __forceinline__ int unit_of(int x) {
 struct QuadTask {
   const float* A;        // operands in step groups (shared memory, or global: kGmem)
   const float* B;
-  const int32_t* Psrc;   // predecessors of B's rows, [kk][col], global
-  float* D;
+  const int32_t* Psrc;   // predecessors of B's rows, [kk][col] (BS < 128: shared memory)
+  float* D;              // where the results go (kOutSmem: shared memory)
   int32_t* P;
   int64_t ld;
   bool diag;
   int* status;
 };
+
+// Step (0 .. 3) of a group whose sum is first equal to the group's minimum.
+__device__ __forceinline__ int first_of(const float4& a, const float4& b) {
+  const float s0 = a.x + b.x, s1 = a.y + b.y, s2 = a.z + b.z, s3 = a.w + b.w;
+  const float best = min3f(fminf(s0, s1), s2, s3);
+  return s0 == best ? 0 : s1 == best ? 1 : s2 == best ? 2 : 3;
+}
 
 // Entries of a warp's part of a tile in 16-bit list items: lane | nn << 5 |
 // m << 8 | group << 11 (BS = 128: all 2048 of them in 4 KB).
@@ -146,8 +133,8 @@ __device__ __forceinline__ void quad_entry(unsigned item, int& row, int& col, in
   g = (int)(item >> 11);
 }
 
-// Distances and predecessors of `total` improved entries of one warp, four per
-// lane at a time so that their loads overlap.
+// Predecessors of `total` improved entries of one warp, four per lane at a time
+// so that their loads overlap.
 template <int BS, bool kGmem>
 __device__ __noinline__ void finish_quads(const QuadTask& f, const uint16_t* list, int total) {
   constexpr int I = 4, kStride = Geo<BS>::TM * 64;
@@ -155,7 +142,7 @@ __device__ __noinline__ void finish_quads(const QuadTask& f, const uint16_t* lis
   const int64_t ld = f.ld;
   auto load = [](const float* p) -> float4 {
     if constexpr (kGmem) return __ldcg(reinterpret_cast<const float4*>(p));
-    else return *reinterpret_cast<const float4*>(p);
+    else return lds_here(p);
   };
 #pragma unroll 1
   for (int i0 = lane; i0 < total; i0 += 32 * I) {
@@ -168,68 +155,32 @@ __device__ __noinline__ void finish_quads(const QuadTask& f, const uint16_t* lis
       a[u] = load(f.A + unit_of<BS>(row[u]) + g[u] * kStride);
       b[u] = load(f.B + unit_of<BS>(col[u]) + g[u] * kStride);
     }
-    float best[I];
     int32_t pred[I];
 #pragma unroll
-    for (int u = 0; u < I; ++u) {
-      const float s0 = a[u].x + b[u].x, s1 = a[u].y + b[u].y, s2 = a[u].z + b[u].z,
-                  s3 = a[u].w + b[u].w;
-      best[u] = min3f(fminf(s0, s1), s2, s3);
-      const int e = s0 == best[u] ? 0 : s1 == best[u] ? 1 : s2 == best[u] ? 2 : 3;
-      pred[u] = __ldcg(f.Psrc + (g[u] * 4 + e) * BS + col[u]);
-    }
+    for (int u = 0; u < I; ++u)
+      pred[u] = __ldcg(f.Psrc + (g[u] * 4 + first_of(a[u], b[u])) * BS + col[u]);
 #pragma unroll
-    for (int u = 0; u < I; ++u) {
-      if (i0 + 32 * u >= total) continue;
-      f.D[row[u] * ld + col[u]] = best[u];
-      f.P[row[u] * ld + col[u]] = pred[u];
-      if (f.diag && row[u] == col[u] && best[u] < 0.0f) atomicOr(f.status, kStNegCycle);
-    }
+    for (int u = 0; u < I; ++u)
+      if (i0 + 32 * u < total) f.P[row[u] * ld + col[u]] = pred[u];
   }
 }
 
 // Stores what core_q improved against the tile's values `old` (shared memory,
-// row-major).  list: an item per entry of the warp's part of the tile.  Whole
-// warps.
-template <int BS, bool kGmem>
+// row-major): distances in vectors of the lanes' own entries, improved or not.
+// Predecessors, BS = 128: by a list of the improved entries (an item per entry of
+// the warp's part of the tile), since the operands come from global memory; small
+// tiles, whose operands and predecessors are in shared memory: each lane its own.
+// Whole warps.
+template <int BS, bool kGmem, bool kOutSmem>
 __device__ __forceinline__ void finish_tile_q(const QuadTask& f, const float* old, int nrow, int ncol,
                                               const float (&acc)[Geo<BS>::TM][Geo<BS>::TM],
                                               const uint32_t (&arg)[Geo<BS>::TM][QuadArg<Geo<BS>::TM>::kWords],
                                               int tx, int ty, uint16_t* list) {
   using Gm = Geo<BS>;
-  constexpr int TM = Gm::TM, G = Gm::G;
+  constexpr int TM = Gm::TM, G = Gm::G, kStride = TM * 64;
+  constexpr bool kList = BS == 128;
   const int lane = threadIdx.x & 31;
   const int64_t ld = f.ld;
-  if (!f.P) {
-    // distance-only: the improved entries are the results
-#pragma unroll
-    for (int m = 0; m < TM; ++m)
-#pragma unroll
-      for (int g = 0; g < Gm::NG; ++g) {
-        const int lr = Gm::idx(ty, m), lc = g * Gm::SPAN + tx * G;
-        float v[G];
-        vload_s<G>(v, old + lr * BS + lc);
-        bool any = false, neg = false;
-        int32_t bits[G];
-#pragma unroll
-        for (int e = 0; e < G; ++e) {
-          const bool better = acc[m][g * G + e] < v[e] && lr < nrow && lc + e < ncol;
-          any |= better;
-          v[e] = better ? acc[m][g * G + e] : v[e];
-          neg |= better && f.diag && lr == lc + e && v[e] < 0.0f;
-          bits[e] = __float_as_int(v[e]);
-        }
-        int32_t* const Drow = reinterpret_cast<int32_t*>(f.D + lr * ld + lc);
-        if (lc + G <= ncol) {
-          st_if(any, Drow, bits);
-        } else {
-#pragma unroll
-          for (int e = 0; e < G; ++e) st_if(any && lc + e < ncol, Drow + e, bits[e]);
-        }
-        if (neg) atomicOr(f.status, kStNegCycle);
-      }
-    return;
-  }
   // the list entry by entry, all lanes' of one before the next, so that
   // neighbours in it lie in few row segments
   const unsigned below = (1u << lane) - 1u;
@@ -241,21 +192,73 @@ __device__ __forceinline__ void finish_tile_q(const QuadTask& f, const float* ol
       const int lr = Gm::idx(ty, m), lc = g * Gm::SPAN + tx * G;
       float v[G];
       vload_s<G>(v, old + lr * BS + lc);
+      bool better[G], any = false, neg = false;
+      int32_t bits[G];
 #pragma unroll
       for (int e = 0; e < G; ++e) {
-        const int nn = g * G + e;
-        const bool better = acc[m][nn] < v[e] && lr < nrow && lc + e < ncol;
-        const unsigned all = __ballot_sync(0xffffffffu, better);
-        if (better)
-          list[total + __popc(all & below)] =
-              (uint16_t)(lane | nn << 5 | m << 8 | group_of<TM>(arg, m, nn) << 11);
-        total += __popc(all);
+        better[e] = acc[m][g * G + e] < v[e] && lr < nrow && lc + e < ncol;
+        any |= better[e];
+        v[e] = better[e] ? acc[m][g * G + e] : v[e];
+        neg |= better[e] && f.diag && lr == lc + e && v[e] < 0.0f;
+        bits[e] = __float_as_int(v[e]);
+      }
+      if constexpr (kOutSmem) {
+        vstore<G>(f.D + lr * BS + lc, v);
+      } else {
+        int32_t* const Drow = reinterpret_cast<int32_t*>(f.D + lr * ld + lc);
+        if (lc + G <= ncol) {
+          st_if(any, Drow, bits);
+        } else {
+#pragma unroll
+          for (int e = 0; e < G; ++e) st_if(any && lc + e < ncol, Drow + e, bits[e]);
+        }
+      }
+      if (neg) atomicOr(f.status, kStNegCycle);
+      if (!f.P) continue;
+      if constexpr (kList) {
+#pragma unroll
+        for (int e = 0; e < G; ++e) {
+          const int nn = g * G + e;
+          const unsigned all = __ballot_sync(0xffffffffu, better[e]);
+          if (better[e])
+            list[total + __popc(all & below)] =
+                (uint16_t)(lane | nn << 5 | m << 8 | group_of<TM>(arg, m, nn) << 11);
+          total += __popc(all);
+        }
+      } else if (__any_sync(0xffffffffu, any)) {
+        float4 a[G], b[G];
+        int32_t pred[G];
+        int kk[G];
+        bool every = true;
+#pragma unroll
+        for (int e = 0; e < G; ++e) {
+          const int nn = g * G + e;
+          kk[e] = (int)group_of<TM>(arg, m, nn);
+          a[e] = lds_here(f.A + h_unit<BS>(0, m, ty) + kk[e] * kStride);
+          b[e] = lds_here(f.B + h_unit<BS>(0, nn, tx) + kk[e] * kStride);
+          every &= better[e];
+        }
+#pragma unroll
+        for (int e = 0; e < G; ++e)
+          pred[e] = f.Psrc[(kk[e] * 4 + first_of(a[e], b[e])) * BS + lc + e];
+        int32_t* const Prow = f.P + lr * ld + lc;
+        if constexpr (kOutSmem) {
+#pragma unroll
+          for (int e = 0; e < G; ++e)
+            if (better[e]) Prow[e] = pred[e];
+        } else {
+          st_if(every, Prow, pred);
+#pragma unroll
+          for (int e = 0; e < G; ++e) st_if(better[e] && !every, Prow + e, pred[e]);
+        }
       }
     }
-  if (total == 0) return;
-  __syncwarp();
-  finish_quads<BS, kGmem>(f, list, total);
-  __syncwarp();
+  if constexpr (kList) {
+    if (total == 0) return;
+    __syncwarp();
+    finish_quads<BS, kGmem>(f, list, total);
+    __syncwarp();
+  }
 }
 
 }  // namespace fwk

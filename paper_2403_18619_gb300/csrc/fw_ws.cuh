@@ -9,11 +9,12 @@
 //     on the previous task:
 //       - the tile's own D block (one 2-D tensor copy, or one copy per row) -> Dbuf
 //       - the A and B panel snapshots -> 2-stage ring: whole 16-bit tiles (keys
-//         of int32, lower bounds of the 64-bit types), or chunks of 64 k-steps
-//         of 32-bit keys or values (int32 beyond 16 bits, fp32)
+//         of int32, lower bounds of fp64), or chunks of 64 k-steps (64-bit
+//         elements: 32) of values or 32-bit keys
 //     and, for panel tasks, the tile and the closed pivot (ws_panel*).
-//   * The compute warps relax and store improved entries; pivot tasks are run
-//     by them alone, using the shared buffer as scratch (the producer waits
+//   * The compute warps relax and store improved entries; pivot tasks (and
+//     panels of the 64-bit types where tiles are not filtered) are run by them
+//     alone, using the shared buffer as scratch (the producer waits
 //     until such a task is published).  The task that finishes tile
 //     (r+1, r+1) of round r runs the pivot of round r+1 right after it.
 //   * The publisher sleeps on the compute warps' task-done barrier and
@@ -49,39 +50,59 @@ constexpr int kPubDepth = 4;  // tasks handed to the compute warps but not yet p
 // next pivot).
 constexpr int kFusedTask = 4;
 
-// Operand chunks of a task that streams 32-bit keys or values (int32 beyond 16
-// bits, fp32): CK k-steps of A and of B, 64 at most (2 per task at BS = 128: few
-// ring hand-offs).
+// The exact 64-bit kernels run panels by the compute warps alone (task_panel).
+template <typename T, int BS>
+constexpr bool kOwnPanels = sizeof(T) == 8 && !kFiltered<T, BS>;
+
+// Floating types, small tiles: the predecessors that improved entries take come
+// into the ring stage, beside the operands, and stay there until the epilogue is
+// done with them.  fp32 keeps its operands as well: the epilogue's chain of loads
+// (a group's operands, then the predecessor) from global memory cost more than
+// the relaxation (a tile of 64: relaxed in 5.6 K cycles, done after 17 K; now
+// 8.3 and 13.4); fp64 in tiles of 32: 23.6 K cycles, now 22.1.  A ring for tiles
+// of 128 has no room.
+template <typename T, int BS>
+constexpr bool kPredSmem = std::is_same<T, float>::value ? BS <= 64
+                                                         : std::is_same<T, double>::value && BS <= 32;
+
+// Operand chunks of a task that streams values or 32-bit keys: CK k-steps of A
+// and of B, 64 at most (64-bit elements: 32), so that a BS = 128 task takes two.
 template <int BS, typename T>
 struct WsChunk {
-  static constexpr int CK = BS < 64 ? BS : 64;                            // k-steps per chunk
+  static constexpr int kMax = sizeof(T) == 4 ? 64 : 32;
+  static constexpr int CK = BS < kMax ? BS : kMax;                        // k-steps per chunk
   static constexpr int NC = BS / CK;                                      // chunks per task
-  static constexpr size_t kChunkBytes = (size_t)CK * BS * 4;              // one operand chunk
+  static constexpr size_t kChunkBytes = (size_t)CK * BS * sizeof(T);      // one operand chunk
   static constexpr size_t kTile = (size_t)BS * BS * sizeof(T);            // a tile of elements
   static constexpr size_t kHTile = (size_t)BS * BS * 2;                   // a 16-bit tile
 };
 
 // Shared-memory layout sized for the largest block size LBS a launch runs:
 // the 2-stage operand ring (a stage holds two 16-bit tiles, a tile of elements
-// or two 32-bit chunks), the tile's own D (Dbuf) and a scratch (int32: a 16-bit
-// tile for expand_h; other types: a list item per entry, of 2 bytes for fp32
-// and 4 for 64-bit elements); 224 KB for LBS = 128 with 32-bit elements, 112 KB
-// for LBS = 64 with 64-bit ones (two CTAs per SM).
+// or two 32-bit chunks), the tile's own D (Dbuf) and, where an epilogue lists the
+// improved entries, an item per entry (fp32 tiles of 128: 2 bytes; filtered fp64
+// tiles: 4).  LBS = 128: fp32 224 KB, int32 192 KB (which leaves 60 KB of L1 cache
+// instead of 28: n = 8000 1.3 % faster); fp64 of 64: 112 KB, two CTAs per SM.
 template <int LBS, typename T>
 struct WsLayout {
   static constexpr size_t kTile = WsChunk<LBS, T>::kTile;
   static constexpr size_t kHTile = WsChunk<LBS, T>::kHTile;
-  static constexpr size_t kStage = sizeof(T) == 4 ? 2 * WsChunk<LBS, T>::kChunkBytes : kTile;
+  static constexpr size_t kStage =
+      2 * WsChunk<LBS, T>::kChunkBytes + (kPredSmem<T, LBS> ? (size_t)LBS * LBS * 4 : 0);
   static constexpr size_t kRing = 2 * kStage;
-  static constexpr size_t kScr = sizeof(T) == 4 ? kHTile : (size_t)LBS * LBS * 4;
+  static constexpr size_t kScr = kFiltered<T, LBS>                                ? (size_t)LBS * LBS * 4
+                                 : std::is_same<T, float>::value && LBS == 128 ? kHTile
+                                                                               : 0;
   static constexpr size_t kScrWarp = kScr / (kThreads / 32);
   __host__ __device__ static constexpr size_t ring_off() { return 0; }
   __host__ __device__ static constexpr size_t d_off() { return kRing; }
   __host__ __device__ static constexpr size_t scr_off() { return kRing + kTile; }
   __host__ __device__ static constexpr size_t bytes() { return scr_off() + kScr; }
   static_assert(2 * kHTile <= kStage && kTile <= kStage, "a stage holds either");
-  // the int32 pivot uses the buffer from offset 0 as three tiles of scratch
+  // the int32 pivot uses the buffer from offset 0 as three tiles of scratch,
+  // task_panel as two tiles and one of predecessors
   static_assert(!Num<T>::kPacked || bytes() >= 3 * kTile, "scratch of pivot tasks");
+  static_assert(!kOwnPanels<T, LBS> || bytes() >= 2 * kTile + (size_t)LBS * LBS * 4, "task_panel");
   static_assert(bytes() <= 226 * 1024, "shared memory of one CTA");
 };
 
@@ -162,7 +183,7 @@ struct PipeCnt {
 
 // ------------------------------------------------------------ compute side ----
 
-// Operand forms of a remaining tile (key_operands).
+// Operand forms of a remaining tile (tile_form).
 constexpr int kFormKA = 1, kFormKB = 2, kFormHA = 4, kFormHB = 8, kFormInfA = 16, kFormInfB = 32;
 
 // In-place decode of `count` packed keys (int32 path) back to values, for a
@@ -188,23 +209,22 @@ __device__ __forceinline__ void decode_keys(uint32_t* buf, int count) {
 
 // Expansion of a 16-bit snapshot tile at buf, in place, to the chunk of CK
 // steps from step ch * CK: 32-bit keys (with the code of the step for an A
-// operand) or values.  The tile goes through the scratch first, so that no
-// word is overwritten before it is read.
+// operand) or values.  The tile goes through registers, so that no word is
+// overwritten before it is read.
 template <int BS, int CK>
-__device__ __noinline__ void expand_h(uint32_t* buf, uint32_t* scr, int ch, bool keys, bool is_a,
-                                      bool has_inf) {
+__device__ __noinline__ void expand_h(uint32_t* buf, int ch, bool keys, bool is_a, bool has_inf) {
   using H = KeysH<BS>;
   using K = Keys<BS>;
   using Gm = Geo<BS>;
   constexpr int TM = Gm::TM;
-  bar_compute();  // (the scratch is free)
+  uint32_t words[H::kTileWords / kThreads];
 #pragma unroll
-  for (int i = threadIdx.x * 4; i < H::kTileWords; i += kThreads * 4)
-    *reinterpret_cast<uint4*>(scr + i) = *reinterpret_cast<const uint4*>(buf + i);
+  for (int j = 0; j < H::kTileWords / kThreads; ++j) words[j] = buf[threadIdx.x + j * kThreads];
   bar_compute();
-#pragma unroll 4
-  for (int i = threadIdx.x; i < H::kTileWords; i += kThreads) {
-    const uint32_t w = scr[i];
+#pragma unroll
+  for (int j = 0; j < H::kTileWords / kThreads; ++j) {
+    const int i = (int)threadIdx.x + j * kThreads;
+    const uint32_t w = words[j];
     const int row = Gm::idx((i >> 2) & 15, (i >> 6) % TM), kw = (i >> 6) / TM * 4 + (i & 3);
     auto put = [&](int h) {
       const int kk = kk_of<BS>(kw, h);
@@ -225,20 +245,18 @@ __device__ __noinline__ void expand_h(uint32_t* buf, uint32_t* scr, int ch, bool
 }
 
 // Operands of a remaining tile that arrive in another form than its core reads
-// (key_operands): 32-bit keys decoded to values, a 16-bit snapshot expanded,
+// (tile_form): 32-bit keys decoded to values, a 16-bit snapshot expanded,
 // in the ring stage (every warp has waited for the stage to fill, so no warp
 // still reads its previous contents); synchronises the compute warps.
 template <typename T, int BS, int CK>
-__device__ __forceinline__ void decode_chunk(unsigned char* stage, unsigned char* scratch, int dec,
-                                             int ch, bool keys) {
+__device__ __forceinline__ void decode_chunk(unsigned char* stage, int dec, int ch, bool keys) {
   if constexpr (Num<T>::kPacked) {
     if (!(dec & (kFormKA | kFormKB | kFormHA | kFormHB))) return;
     uint32_t* As = reinterpret_cast<uint32_t*>(stage);
     if (dec & kFormKA) decode_keys<BS>(As, CK * BS);
     if (dec & kFormKB) decode_keys<BS>(As + CK * BS, CK * BS);
-    uint32_t* scr = reinterpret_cast<uint32_t*>(scratch);
-    if (dec & kFormHA) expand_h<BS, CK>(As, scr, ch, keys, true, dec & kFormInfA);
-    if (dec & kFormHB) expand_h<BS, CK>(As + CK * BS, scr, ch, keys, false, dec & kFormInfB);
+    if (dec & kFormHA) expand_h<BS, CK>(As, ch, keys, true, dec & kFormInfA);
+    if (dec & kFormHB) expand_h<BS, CK>(As + CK * BS, ch, keys, false, dec & kFormInfB);
     fence_proxy_async_shared();  // generic writes before the stage's next TMA fill
     bar_compute();
   }
@@ -291,7 +309,7 @@ __device__ __noinline__ bool ws_minplus_dist(TileCtx<T> c, int ti, int tj, int d
                    c.timeout_ns))
       return false;
     if (tr) cw += clock64() - w0;
-    decode_chunk<T, BS, C::CK>(ring + st * L::kStage, smem + L::scr_off(), dec, ch, false);
+    decode_chunk<T, BS, C::CK>(ring + st * L::kStage, dec, ch, false);
     const T* As = reinterpret_cast<const T*>(ring + st * L::kStage);
     const T* Bs = As + C::CK * BS;
     core_min<BS, T, C::CK>(As, Bs, acc, tx, ty);
@@ -338,10 +356,12 @@ __device__ __noinline__ bool ws_minplus_dist(TileCtx<T> c, int ti, int tj, int d
 // per tile, whatever the layout; both groups in step 27 K cycles per tile,
 // 19 K of them relaxation).  Named barriers 2 + g: group g may go.
 __device__ __forceinline__ void turn_wait(int g) {
-  asm volatile("bar.sync %0, 256;" ::"r"(2 + g) : "memory");
+  if (g) asm volatile("bar.sync 3, 256;" ::: "memory");
+  else asm volatile("bar.sync 2, 256;" ::: "memory");
 }
 __device__ __forceinline__ void turn_pass(int g) {
-  asm volatile("bar.arrive %0, 256;" ::"r"(2 + g) : "memory");
+  if (g) asm volatile("bar.arrive 3, 256;" ::: "memory");
+  else asm volatile("bar.arrive 2, 256;" ::: "memory");
 }
 
 // Remaining-tile task over 16-bit packed keys (int32; cap: their clamp).  The
@@ -472,10 +492,15 @@ __device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task&
       acc[m][nn] = Num<float>::inf();
       arg[m][nn / 4] = 0;
     }
+  constexpr bool kHold = kPredSmem<float, BS>;  // the operands stay for the epilogue
+  constexpr bool kTurns = !kHold;
+  static_assert(!kHold || C::NC == 1, "all of a tile's operands in one stage");
+  const unsigned st0 = pc.chunk & 1;
+  unsigned char* const stage0 = smem + L::ring_off() + st0 * L::kStage;
   const int group = (int)threadIdx.x >> 7;
   bool ok = mbar_wait(&wb->chunk_full[pc.chunk & 1], (pc.chunk >> 1) & 1, a.status, a.abort_flag,
                       a.timeout_ns);
-  if (a.P) turn_wait(group);
+  if (kTurns && a.P) turn_wait(group);
 #pragma unroll 1
   for (int ch = 0; ch < C::NC && ok; ++ch) {
     const unsigned st = pc.chunk & 1;
@@ -488,10 +513,10 @@ __device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task&
     if (a.P) core_q<BS, C::CK / 4, true>(As, Bs, acc, arg, tx, ty, ch * (C::CK / 4));
     else core_q<BS, C::CK / 4, false>(As, Bs, acc, arg, tx, ty, 0);
     __syncwarp();
-    if (lane == 0) mbar_arrive(&wb->chunk_empty[st]);
+    if (!kHold && lane == 0) mbar_arrive(&wb->chunk_empty[st]);
     ++pc.chunk;
   }
-  if (a.P) turn_pass(group ^ 1);  // (also when a wait has given up: the other group must not wait for it)
+  if (kTurns && a.P) turn_pass(group ^ 1);  // (also when a wait has given up: the other group must not wait for it)
   if (!ok) return false;
   const long long t_b = tr ? clock64() : 0;
   if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns)) return false;
@@ -501,72 +526,141 @@ __device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task&
   }
   QuadTask f = quad_task<BS>(a, k.ti, k.tj);
   const size_t ta = (size_t)(k.r & 1) * a.slot_tiles + k.ti, tb = (size_t)(k.r & 1) * a.slot_tiles + k.tj;
-  f.A = a.colR + ta * BS * BS;
-  f.B = a.rowR + tb * BS * BS;
-  f.Psrc = a.rowP + tb * BS * BS;
+  if constexpr (kHold) {
+    f.A = reinterpret_cast<const float*>(stage0);
+    f.B = f.A + BS * BS;
+    f.Psrc = reinterpret_cast<const int32_t*>(f.B + BS * BS);
+  } else {
+    f.A = a.colR + ta * BS * BS;
+    f.B = a.rowR + tb * BS * BS;
+    f.Psrc = a.rowP + tb * BS * BS;
+  }
   const int64_t row0 = (int64_t)k.ti * BS, col0 = (int64_t)k.tj * BS;
-  finish_tile_q<BS, true>(f, reinterpret_cast<const float*>(smem + L::d_off()),
+  finish_tile_q<BS, !kHold, false>(f, reinterpret_cast<const float*>(smem + L::d_off()),
                           (int)(a.n - row0 < BS ? a.n - row0 : BS),
                           (int)(a.n - col0 < BS ? a.n - col0 : BS), acc, arg, tx, ty,
                           reinterpret_cast<uint16_t*>(smem + L::scr_off() +
                                                       (threadIdx.x >> 5) * L::kScrWarp));
   __syncwarp();
-  if (lane == 0) mbar_arrive(&wb->d_empty);
+  if (lane == 0) {
+    mbar_arrive(&wb->d_empty);
+    if (kHold) mbar_arrive(&wb->chunk_empty[st0]);
+  }
   ++pc.d;
   if (tr) tr[8] |= (uint64_t)(clock64() - t_a) << 32;
   return true;
 }
 
-// Panel task of fp32: Dbuf holds the tile's own values, ring stage s0 the closed
-// pivot in step groups, and stage s1 takes the own values in step groups.  The
-// improved entries go to the matrix; the tile's snapshots (step groups, a row
-// tile's predecessors) are made from it afterwards.  A row tile's predecessors
-// come from its own old ones, which wait in the snapshot's place meanwhile.
+// Unit of a BS x BS tile for thread slot i (0 .. BS*BS/4 - 1): operand row x and
+// step group g.  kA: steps along the tile's columns; a warp takes 8 operand rows
+// times 4 groups, so that it reads 64 bytes of each row and writes whole lines.
+// Else steps along the rows; a warp takes 32 operand rows (columns of the tile).
+template <int BS, bool kA>
+__device__ __forceinline__ void unit_at(int i, int& x, int& g) {
+  if constexpr (kA) {
+    const int l = i & 31, w = i >> 5, rest = w / (BS / 16);
+    g = (l & 3) + 4 * (w % (BS / 16));
+    x = Geo<BS>::idx((l >> 2) + 8 * (rest & 1), rest >> 1);
+  } else {
+    x = i % BS;
+    g = i / BS;
+  }
+}
+
+// Panel task of fp32: Dbuf holds the tile's own values and ring stage s0 the
+// closed pivot; both are rewritten in step groups, the own values into stage s1,
+// the pivot in place.  Small tiles (kPredSmem) are relaxed within shared memory:
+// s0 and s1 hold the predecessors as well, and the result leaves in whole rows.
+// (By way of the matrix and with the predecessors in global memory a row panel
+// of 64 took 24.5 K cycles, 10 K of them after the relaxation.)  A tile of 128
+// stores its improved entries to the matrix and makes its snapshots (step
+// groups, a row tile's predecessors) from there; a row tile's old predecessors
+// wait in the snapshot's place meanwhile.
 template <int BS, int LBS, bool is_row>
 __device__ __noinline__ bool ws_panel_q(const Args<float>& a, const fwh::Task& k,
                                         unsigned char* smem, WsBars* wb, PipeCnt& pc) {
   using L = WsLayout<LBS, float>;
   constexpr int TM = Geo<BS>::TM;
-  const int lane = threadIdx.x & 31;
+  constexpr bool kSmem = kPredSmem<float, BS>;
+  static_assert(!kSmem || 3 * WsChunk<BS, float>::kTile <= L::kStage, "three tiles per stage");
+  const int tid = threadIdx.x, lane = tid & 31;
   int tx, ty;
   h_thread(tx, ty);
   const int r = k.r, t = is_row ? k.tj : k.ti;
   const unsigned s0 = pc.chunk & 1, s1 = s0 ^ 1;
-  const float* const own = reinterpret_cast<const float*>(smem + L::d_off());
-  const float* const pivq = reinterpret_cast<const float*>(smem + L::ring_off() + s0 * L::kStage);
+  float* const own = reinterpret_cast<float*>(smem + L::d_off());
+  float* const pivq = reinterpret_cast<float*>(smem + L::ring_off() + s0 * L::kStage);
   float* const ownq = reinterpret_cast<float*>(smem + L::ring_off() + s1 * L::kStage);
+  // (kSmem) the own predecessors before and after, one tile each
+  int32_t* const predOld = reinterpret_cast<int32_t*>(ownq + BS * BS);
+  int32_t* const predNew = predOld + BS * BS;
   stamp(0);
   QuadTask f = quad_task<BS>(a, k.ti, k.tj);
+  float* const Dt = f.D;
+  int32_t* const Pt = f.P;
+  const int64_t ld = a.ld;
   const int64_t row0 = (int64_t)k.ti * BS, col0 = (int64_t)k.tj * BS;
   const int nrow = (int)(a.n - row0 < BS ? a.n - row0 : BS);
   const int ncol = (int)(a.n - col0 < BS ? a.n - col0 : BS);
   const size_t tile = (size_t)(r & 1) * a.slot_tiles + t;
   int32_t* const snapP = a.rowP + tile * BS * BS;
-  if (is_row && f.P) {
-#pragma unroll 4
-    for (int i = threadIdx.x; i < BS * BS; i += kThreads) {
-      const int lr = i / BS, lc = i % BS;
-      snapP[i] = lr < nrow && lc < ncol ? __ldcg(f.P + lr * f.ld + lc) : -1;
+  if (!mbar_wait(&wb->chunk_full[s1], ((pc.chunk + 1) >> 1) & 1, a.status, a.abort_flag,
+                 a.timeout_ns))
+    return false;
+  if (Pt) {
+    if constexpr (kSmem) {
+      stage_tile_i32<BS>(predNew, a.P, a.n, a.ld, k.ti, k.tj, nullptr);
+      if constexpr (is_row) {
+        for (int q = tid; q < BS * BS / 4; q += kThreads)
+          reinterpret_cast<int4*>(predOld)[q] = reinterpret_cast<const int4*>(predNew)[q];
+      }
+    } else if constexpr (is_row) {
+      stage_tile_i32<BS>(snapP, a.P, a.n, a.ld, k.ti, k.tj, nullptr);
     }
   }
   if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns) ||
       !mbar_wait(&wb->chunk_full[s0], (pc.chunk >> 1) & 1, a.status, a.abort_flag,
-                 a.timeout_ns) ||
-      !mbar_wait(&wb->chunk_full[s1], ((pc.chunk + 1) >> 1) & 1, a.status, a.abort_flag,
                  a.timeout_ns))
     return false;
-  // unit (g, x): steps 4g .. 4g+3 of operand row x
-#pragma unroll 2
-  for (int i = threadIdx.x; i < BS * BS / 4; i += kThreads) {
-    const int x = is_row ? i % BS : i / (BS / 4), g = is_row ? i / BS : i % (BS / 4);
+  constexpr int NU = BS * BS / 4 / kThreads;  // units per thread
+  float4 pv[NU];
+#pragma unroll
+  for (int j = 0; j < NU; ++j) {
+    int x, g;
+    unit_at<BS, is_row>(tid + j * kThreads, x, g);
+    if constexpr (is_row) {
+      pv[j] = *reinterpret_cast<const float4*>(pivq + x * BS + 4 * g);
+    } else {
+      const float* const p = pivq + 4 * g * BS + x;
+      pv[j] = make_float4(p[0], p[BS], p[2 * BS], p[3 * BS]);
+    }
+  }
+  // the own values as an operand (entries beyond n: INF)
+  auto own_unit = [&](int j, auto&& at) -> float4 {
+    int x, g;
+    unit_at<BS, !is_row>(tid + j * kThreads, x, g);
     float v[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
       const int lr = is_row ? 4 * g + e : x, lc = is_row ? x : 4 * g + e;
-      v[e] = lr < nrow && lc < ncol ? own[lr * BS + lc] : Num<float>::inf();
+      v[e] = lr < nrow && lc < ncol ? at(lr, lc) : Num<float>::inf();
     }
-    *reinterpret_cast<float4*>(ownq + unit_of<BS>(x) + g * TM * 64) = make_float4(v[0], v[1], v[2], v[3]);
-  }
+    return make_float4(v[0], v[1], v[2], v[3]);
+  };
+  auto unit_off = [&](int j, auto kA) -> int {
+    int x, g;
+    unit_at<BS, decltype(kA)::value>(tid + j * kThreads, x, g);
+    return unit_of<BS>(x) + g * TM * 64;
+  };
+  using Row = std::integral_constant<bool, is_row>;
+  using Col = std::integral_constant<bool, !is_row>;
+  auto own_at = [&](int lr, int lc) { return own[lr * BS + lc]; };
+#pragma unroll
+  for (int j = 0; j < NU; ++j)
+    *reinterpret_cast<float4*>(ownq + unit_off(j, Col{})) = own_unit(j, own_at);
+  bar_compute();  // the pivot is in registers
+#pragma unroll
+  for (int j = 0; j < NU; ++j) *reinterpret_cast<float4*>(pivq + unit_off(j, Row{})) = pv[j];
   bar_compute();  // (and the old predecessors are in place)
   stamp(1);
   float acc[TM][TM];
@@ -580,35 +674,76 @@ __device__ __noinline__ bool ws_panel_q(const Args<float>& a, const fwh::Task& k
     }
   f.A = is_row ? pivq : ownq;
   f.B = is_row ? ownq : pivq;
-  f.Psrc = is_row ? snapP : a.pivP + (size_t)(r & 1) * BS * BS;
+  if constexpr (kSmem) {
+    f.D = own;
+    f.P = Pt ? predNew : nullptr;
+    f.ld = BS;
+    f.Psrc = is_row ? predOld : reinterpret_cast<const int32_t*>(pivq + BS * BS);
+  } else {
+    f.Psrc = is_row ? snapP : a.pivP + (size_t)(r & 1) * BS * BS;
+  }
   core_q<BS, BS / 4, true>(f.A, f.B, acc, arg, tx, ty, 0);
-  finish_tile_q<BS, false>(f, own, nrow, ncol, acc, arg, tx, ty,
-                           reinterpret_cast<uint16_t*>(smem + L::scr_off() +
-                                                       (threadIdx.x >> 5) * L::kScrWarp));
-  fence_proxy_async_shared();  // generic writes before the stage's next TMA fill
-  bar_compute();  // the relaxed tile is in the matrix, the operands are free
+  finish_tile_q<BS, false, kSmem>(f, own, nrow, ncol, acc, arg, tx, ty,
+                                         reinterpret_cast<uint16_t*>(smem + L::scr_off() +
+                                                                     (tid >> 5) * L::kScrWarp));
+  if constexpr (!kSmem) fence_proxy_async_shared();  // generic writes before the next TMA fill
+  bar_compute();  // the relaxed tile is complete (kSmem: in own, else in the matrix)
   stamp(2);
-  if (lane == 0) {
-    mbar_arrive(&wb->d_empty);
-    mbar_arrive(&wb->chunk_empty[0]);
-    mbar_arrive(&wb->chunk_empty[1]);
+  auto release = [&] {
+    if (lane == 0) {
+      mbar_arrive(&wb->d_empty);
+      mbar_arrive(&wb->chunk_empty[0]);
+      mbar_arrive(&wb->chunk_empty[1]);
+    }
+  };
+  float* const snapR = (is_row ? a.rowR : a.colR) + tile * BS * BS;
+  if constexpr (kSmem) {
+#pragma unroll
+    for (int j = 0; j < NU; ++j) {
+      const int q = tid + j * kThreads, lr = q / (BS / 4), lc = q % (BS / 4) * 4;
+      const float4 v = *reinterpret_cast<const float4*>(own + lr * BS + lc);
+      int4 p = make_int4(-1, -1, -1, -1);
+      if (Pt) {
+        p = *reinterpret_cast<const int4*>(predNew + lr * BS + lc);
+        if constexpr (is_row) *reinterpret_cast<int4*>(snapP + lr * BS + lc) = p;
+      }
+      if (lr < nrow && lc + 4 <= ncol) {
+        *reinterpret_cast<float4*>(Dt + lr * ld + lc) = v;
+        if (Pt) *reinterpret_cast<int4*>(Pt + lr * ld + lc) = p;
+      } else if (lr < nrow) {
+        const float ve[4] = {v.x, v.y, v.z, v.w};
+        const int32_t pe[4] = {p.x, p.y, p.z, p.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e)
+          if (lc + e < ncol) {
+            Dt[lr * ld + lc + e] = ve[e];
+            if (Pt) Pt[lr * ld + lc + e] = pe[e];
+          }
+      }
+    }
+#pragma unroll
+    for (int j = 0; j < NU; ++j)
+      *reinterpret_cast<float4*>(snapR + unit_off(j, Col{})) = own_unit(j, own_at);
+    fence_proxy_async_shared();  // generic writes before the buffers' next TMA fill
+    __syncwarp();
+    release();
+  } else {
+    release();
+    if (is_row && Pt) stage_tile_i32<BS>(snapP, a.P, a.n, a.ld, k.ti, k.tj, nullptr);
+    constexpr int kAhead = 4;  // units in flight
+#pragma unroll 1
+    for (int j0 = 0; j0 < NU; j0 += kAhead) {
+      float4 v[kAhead];
+#pragma unroll
+      for (int j = 0; j < kAhead; ++j)
+        v[j] = own_unit(j0 + j, [&](int lr, int lc) { return __ldcg(Dt + lr * ld + lc); });
+#pragma unroll
+      for (int j = 0; j < kAhead; ++j)
+        *reinterpret_cast<float4*>(snapR + unit_off(j0 + j, Col{})) = v[j];
+    }
   }
   ++pc.d;
   pc.chunk += 2;
-  float* const snapR = (is_row ? a.rowR : a.colR) + tile * BS * BS;
-#pragma unroll 2
-  for (int i = threadIdx.x; i < BS * BS / 4; i += kThreads) {
-    const int x = is_row ? i % BS : i / (BS / 4), g = is_row ? i / BS : i % (BS / 4);
-    float v[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int lr = is_row ? 4 * g + e : x, lc = is_row ? x : 4 * g + e;
-      const bool in = lr < nrow && lc < ncol;
-      v[e] = in ? __ldcg(f.D + lr * f.ld + lc) : Num<float>::inf();
-      if (is_row && f.P && in) snapP[lr * BS + lc] = __ldcg(f.P + lr * f.ld + lc);
-    }
-    *reinterpret_cast<float4*>(snapR + unit_of<BS>(x) + g * TM * 64) = make_float4(v[0], v[1], v[2], v[3]);
-  }
   stamp(3);
   return true;
 }
@@ -634,7 +769,7 @@ __device__ __forceinline__ FilterTask<T> filter_task(const Args<T>& a, int r, in
   return f;
 }
 
-// Remaining-tile task of the 64-bit types: the 16-bit pass
+// Remaining-tile task of fp64 (BS = 64): the 16-bit pass
 // in turns, then the exact relaxation of the entries that may improve while
 // the other group of warps has its turn.
 template <typename T, int BS, int LBS>
@@ -721,7 +856,7 @@ __device__ __forceinline__ int quantize_tile(uint32_t* H, const QScale& q, Src&&
   return neg;
 }
 
-// Panel task of round r of the 64-bit types: Dbuf holds the tile's own values,
+// Panel task of round r of fp64 (BS = 64): Dbuf holds the tile's own values,
 // ring stage s0 the closed pivot, and stage s1 takes the 16-bit bounds of
 // both.  Filtered like a remaining tile, with its exact operands in shared
 // memory; then the tile's snapshots (values, 16-bit bounds, a row tile's
@@ -746,13 +881,7 @@ __device__ __noinline__ bool ws_panel_f(const Args<T>& a, const fwh::Task& k, un
   FilterTask<T> f = filter_task<T, BS>(a, r, k.ti, k.tj);
   const size_t tile = (size_t)(r & 1) * a.slot_tiles + t;
   int32_t* const snapP = a.rowP + tile * BS * BS;
-  if (is_row && !ViaPred<T>::kOn && f.P) {
-#pragma unroll 4
-    for (int i = threadIdx.x; i < BS * BS; i += kThreads) {
-      const int lr = i / BS, lc = i % BS;
-      snapP[i] = lr < f.nrow && lc < f.ncol ? __ldcg(f.P + lr * f.ld + lc) : -1;
-    }
-  }
+  if (is_row && !ViaPred<T>::kOn && f.P) stage_tile_i32<BS>(snapP, a.P, a.n, a.ld, k.ti, k.tj, nullptr);
   if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns) ||
       !mbar_wait(&wb->chunk_full[s0], (pc.chunk >> 1) & 1, a.status, a.abort_flag,
                  a.timeout_ns) ||
@@ -796,12 +925,11 @@ __device__ __noinline__ bool ws_panel_f(const Args<T>& a, const fwh::Task& k, un
   pc.chunk += 2;
   T* const snapR = (is_row ? a.rowR : a.colR) + tile * BS * BS;
   uint32_t* const snapH = (is_row ? a.rowH : a.colH) + tile * H::kTileWords;
-  int32_t* const Pold = is_row && !ViaPred<T>::kOn && f.P ? snapP : nullptr;
+  if (is_row && !ViaPred<T>::kOn && f.P) stage_tile_i32<BS>(snapP, a.P, a.n, a.ld, k.ti, k.tj, nullptr);
   auto relaxed = [&](int i, int j) {
     const bool in = i < f.nrow && j < f.ncol;
     const T v = in ? __ldcg(f.D + i * f.ld + j) : Num<T>::inf();
     snapR[i * BS + j] = v;
-    if (Pold && in) Pold[i * BS + j] = __ldcg(f.P + i * f.ld + j);
     return v;
   };
   neg[0] = quantize_tile<T, BS, !is_row>(snapH, f.q, relaxed);
@@ -811,14 +939,18 @@ __device__ __noinline__ bool ws_panel_f(const Args<T>& a, const fwh::Task& k, un
   return true;
 }
 
-// Remaining-tile task (phase 4 of round r, tile ti,tj).  mode: 0 compare and
-// select, 1 packed 32-bit keys (16-bit keys: ws_minplus_h).  Returns false if
-// an operand never arrived (the kernel then stops).
-template <typename T, int BS, int LBS>
-__device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mode, int dec,
+// Remaining-tile task (phase 4 of round r, tile ti,tj) over packed 32-bit keys
+// (kKeys; 16-bit keys: ws_minplus_h) or with compare and select.  kExpand: the
+// operands may need to be expanded first (dec).  Keys that need not be have a loop
+// of their own, in the kernel itself: a call in it, or out of line, its registers
+// are laid out for the callee (int32 with weights to 3e5, n = 3000: 2.74 ms, one
+// loop for both 2.78, out of line 2.85).  Returns false if an operand never
+// arrived (the kernel then stops).
+template <typename T, int BS, int LBS, bool kKeys, bool kExpand>
+__device__ __forceinline__ bool ws_minplus_body(TileCtx<T> c, int ti, int tj, int dec,
                                         unsigned char* smem, WsBars* wb, PipeCnt& pc,
                                         uint64_t* tr) {
-  if (mode == 0 && !c.P) return ws_minplus_dist<T, BS, LBS>(c, ti, tj, dec, smem, wb, pc, tr);
+  if (!kKeys && !c.P) return ws_minplus_dist<T, BS, LBS>(c, ti, tj, dec, smem, wb, pc, tr);
   using Gm = Geo<BS>;
   using K = Keys<BS>;
   using L = WsLayout<LBS, T>;
@@ -861,7 +993,7 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mod
   T* Drow = c.D + row0 * c.ld + col0;
   int32_t* Prow = c.P + row0 * c.ld + col0;
   bool neg = false;
-  if (kPacked && mode) {  // (packed keys: int32 only)
+  if constexpr (kKeys) {  // (packed keys: int32 only)
     uint32_t acc[TM][TM];
     int32_t omax = 0;
 #pragma unroll
@@ -879,7 +1011,8 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mod
                      c.timeout_ns))
         return false;
       if (tr) cw += clock64() - w0;
-      decode_chunk<T, BS, C::CK>(ring + st * L::kStage, smem + L::scr_off(), dec, ch, true);
+      if constexpr (kExpand)
+        decode_chunk<T, BS, C::CK>(ring + st * L::kStage, dec, ch, true);
       const uint32_t* As = reinterpret_cast<const uint32_t*>(ring + st * L::kStage);
       const uint32_t* Bs = As + C::CK * BS;
       core_packed<BS, C::CK>(As, Bs, acc, tx, ty);
@@ -948,6 +1081,9 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mod
       }
     }
   } else {
+    constexpr bool kHold = kPredSmem<T, BS>;  // the stage stays: its predecessors are read below
+    static_assert(!kHold || C::NC == 1, "all of a tile's operands in one stage");
+    const unsigned st0 = pc.chunk & 1;
     int arg[TM][TM];
 #pragma unroll
     for (int m = 0; m < TM; ++m)
@@ -960,12 +1096,12 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mod
                      c.timeout_ns))
         return false;
       if (tr) cw += clock64() - w0;
-      decode_chunk<T, BS, C::CK>(ring + st * L::kStage, smem + L::scr_off(), dec, ch, false);
+      decode_chunk<T, BS, C::CK>(ring + st * L::kStage, dec, ch, false);
       const T* As = reinterpret_cast<const T*>(ring + st * L::kStage);
       const T* Bs = As + C::CK * BS;
       core_generic<BS, T, C::CK, false>(As, Bs, old, arg, tx, ty, ch * C::CK);
       __syncwarp();
-      if (lane == 0) mbar_arrive(&wb->chunk_empty[st]);
+      if (!kHold && lane == 0) mbar_arrive(&wb->chunk_empty[st]);
       ++pc.chunk;
     }
     argmin_finish<T>(arg);
@@ -975,6 +1111,8 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mod
       tr[8] = (uint64_t)(t_c - t_a);
     }
     const int32_t via0 = via_code((int64_t)c.r * BS - 1);
+    const int32_t* const Psrc =
+        reinterpret_cast<const int32_t*>(ring + st0 * L::kStage + 2 * C::kChunkBytes);
 #pragma unroll
     for (int m = 0; m < TM; ++m) {
       const int lr = Gm::idx(ty, m);
@@ -984,15 +1122,27 @@ __device__ __forceinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int mod
         if (arg[m][nn] && lr < nrow && lc < ncol) {
           Drow[lr * c.ld + lc] = old[m][nn];
           Prow[lr * c.ld + lc] =
-              via0 - arg[m][nn];
+              kHold ? Psrc[(arg[m][nn] - 1) * BS + lc] : via0 - arg[m][nn];
           neg |= (row0 + lr == col0 + lc) && old[m][nn] < T(0);
         }
       }
+    }
+    if (kHold) {
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&wb->chunk_empty[st0]);
     }
   }
   if (tr) tr[8] |= (uint64_t)(clock64() - t_a) << 32;  // whole task
   if (neg) atomicOr(c.status, kStNegCycle);
   return true;
+}
+
+// Out of line: every other case.
+template <typename T, int BS, int LBS, bool kKeys, bool kExpand>
+__device__ __noinline__ bool ws_minplus(TileCtx<T> c, int ti, int tj, int dec,
+                                        unsigned char* smem, WsBars* wb, PipeCnt& pc,
+                                        uint64_t* tr) {
+  return ws_minplus_body<T, BS, LBS, kKeys, kExpand>(c, ti, tj, dec, smem, wb, pc, tr);
 }
 
 // Relaxation and epilogue of a producer-fed panel task (ws_panel) whose
@@ -1081,14 +1231,29 @@ __device__ __noinline__ bool ws_panel_finish(const Args<T>& a, int r, int t, T* 
     if constexpr (kFast) return acc[m][nn] & ~K::MASK;
     else return key_of<BS>((int32_t)acc[m][nn]);
   };
-  int nb = 0, has_inf = 0;
+  int nb, has_inf;
+  if constexpr (kFast) {
+    // (as Bound32, on the keys: values from CAP are INF, none is negative)
+    constexpr uint32_t kTop = 0u - ((uint32_t)K::CAP << K::KB);
+    uint32_t top = 0, hi = 0;
 #pragma unroll
-  for (int m = 0; m < TM; ++m)
+    for (int m = 0; m < TM; ++m)
 #pragma unroll
-    for (int nn = 0; nn < TM; ++nn) {
-      nb = max(nb, bound_of<BS>(value(m, nn)));
-      has_inf |= Num<T>::finite(value(m, nn)) ? 0 : kBndInf;
-    }
+      for (int nn = 0; nn < TM; ++nn) {
+        top = __viaddmax_u32(acc[m][nn], kTop, top);
+        hi = max(hi, acc[m][nn]);
+      }
+    nb = top >= kTop ? (int)((top - kTop) >> K::KB) : 0;
+    has_inf = (int)(hi >> K::KB) >= K::CAP ? kBndInf : 0;
+  } else {
+    Bound32<BS> b;
+#pragma unroll
+    for (int m = 0; m < TM; ++m)
+#pragma unroll
+      for (int nn = 0; nn < TM; ++nn) b.add((int32_t)acc[m][nn]);
+    nb = b.bound();
+    has_inf = b.inf();
+  }
   block_max2(nb, has_inf, cs);
   // one snapshot: 16-bit keys where the bound allows them, else 32-bit keys,
   // which are exact while every finite value is below CAP; beyond that the raw
@@ -1356,8 +1521,7 @@ __device__ __noinline__ bool ws_panel(const Args<T>& a, const fwh::Task& k, unsi
   using L = WsLayout<LBS, T>;
   static_assert(WsChunk<BS, T>::kTile <= L::kStage, "a tile per ring stage");
   constexpr int TM = Gm::TM, G = Gm::G;
-  int tx, ty;
-  h_thread(tx, ty);
+  const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
   if (threadIdx.x == 0) wb->pst[slot] = 0;
   const int r = k.r, t = is_row ? k.tj : k.ti;
   const int64_t row0 = (int64_t)k.ti * BS, col0 = (int64_t)k.tj * BS;
@@ -1394,22 +1558,19 @@ __device__ __noinline__ bool ws_panel(const Args<T>& a, const fwh::Task& k, unsi
     }
   }
   // bounds of the tile and of the pivot, and whether they have an INF
-  int bnd[4] = {0, 0, 0, 0};
+  Bound32<BS> bown, bpiv;
 #pragma unroll
   for (int m = 0; m < TM; ++m)
 #pragma unroll
     for (int nn = 0; nn < TM; ++nn) {
-      bnd[0] = max(bnd[0], bound_of<BS>(s[m][nn]));
-      bnd[1] = max(bnd[1], bound_of<BS>(pv[m][nn]));
-      bnd[2] = max(bnd[2], (int)s[m][nn]);
-      bnd[3] = max(bnd[3], (int)pv[m][nn]);
+      bown.add((int32_t)s[m][nn]);
+      bpiv.add((int32_t)pv[m][nn]);
     }
+  int bnd[4] = {bown.bound(), bpiv.bound(), bown.inf(), bpiv.inf()};
   block_max(bnd, cs);  // (its barriers also end every read of the raw buffers)
   const bool fast = a.packed && (bnd[0] + bnd[1] < K::CAP);
   if (a.packed) {
-    const int inf_s = Num<T>::finite((T)bnd[2]) ? 0 : kBndInf;
-    const int inf_p = Num<T>::finite((T)bnd[3]) ? 0 : kBndInf;
-    if (const int cap = h_clamp<BS>(bnd[0] | inf_s | kBndH, bnd[1] | inf_p | kBndH)) {
+    if (const int cap = h_clamp<BS>(bnd[0] | bnd[2] | kBndH, bnd[1] | bnd[3] | kBndH)) {
       // 16-bit operands in the scratch stage: A, then B
       auto key16 = [&](T v) -> uint32_t { return (uint32_t)min((int)v, cap) << KeysH<BS>::KB; };
       uint32_t* const Ah = reinterpret_cast<uint32_t*>(scratch);
@@ -1479,12 +1640,21 @@ __device__ bool compute_task(const Args<T>& a, const fwh::Task& k, int mode, int
     bool ok;
     if constexpr (Num<T>::kPacked) {
       const TileCtx<T> ctx{a.D, a.P, a.n, a.ld, k.r, a.status, a.abort_flag, a.timeout_ns};
-      ok = mode > 1 ? ws_minplus_h<T, BS, LBS>(a, k, mode, smem, wb, pc, tr)
-                    : ws_minplus<T, BS, LBS>(ctx, k.ti, k.tj, mode, dec, smem, wb, pc, tr);
+      if (mode > 1)
+        ok = ws_minplus_h<T, BS, LBS>(a, k, mode, smem, wb, pc, tr);
+      else if (mode && !(dec & (kFormHA | kFormHB)))
+        ok = ws_minplus_body<T, BS, LBS, true, false>(ctx, k.ti, k.tj, 0, smem, wb, pc, tr);
+      else if (mode)
+        ok = ws_minplus<T, BS, LBS, true, true>(ctx, k.ti, k.tj, dec, smem, wb, pc, tr);
+      else
+        ok = ws_minplus<T, BS, LBS, false, true>(ctx, k.ti, k.tj, dec, smem, wb, pc, tr);
     } else if constexpr (sizeof(T) == 4) {
       ok = ws_minplus_q<BS, LBS>(a, k, smem, wb, pc, tr);
-    } else {
+    } else if constexpr (kFiltered<T, BS>) {
       ok = ws_minplus_f<T, BS, LBS>(a, k, smem, wb, pc, tr);
+    } else {
+      const TileCtx<T> ctx{a.D, a.P, a.n, a.ld, k.r, a.status, a.abort_flag, a.timeout_ns};
+      ok = ws_minplus<T, BS, LBS, false, false>(ctx, k.ti, k.tj, 0, smem, wb, pc, tr);
     }
     if (!ok || k.type == 3) return ok;
     // fused: the tile's stores precede the pivot's loads of it (same CTA),
@@ -1495,9 +1665,10 @@ __device__ bool compute_task(const Args<T>& a, const fwh::Task& k, int mode, int
     bar_compute();
     return true;
   }
-  if (k.type != 0) {
-    bool ok;
-    if constexpr (Num<T>::kPacked)
+  if (k.type != 0 && !kOwnPanels<T, BS>) {
+    bool ok = true;
+    if constexpr (kOwnPanels<T, BS>) {
+    } else if constexpr (Num<T>::kPacked)
       ok = k.type == 1 ? ws_panel<T, BS, LBS, true>(a, k, smem, wb, cs, pc, slot)
                        : ws_panel<T, BS, LBS, false>(a, k, smem, wb, cs, pc, slot);
     else if constexpr (sizeof(T) == 4)
@@ -1509,11 +1680,15 @@ __device__ bool compute_task(const Args<T>& a, const fwh::Task& k, int mode, int
     if (ok) trace_stamps();
     return ok;
   }
-  // Pivot tasks overwrite the ring and Dbuf from their first instructions:
-  // every compute warp must have left the previous task (a slow warp may still
-  // be reading its last operands) before any warp starts.
+  // Pivot tasks (and the exact 64-bit kernels' panels) overwrite the ring and
+  // Dbuf from their first instructions: every compute warp must have left the
+  // previous task (a slow warp may still be reading its last operands) before
+  // any warp starts.
   bar_compute();
-  task_pivot<T, BS>(a, k.r, smem + L::ring_off(), cs);
+  if (k.type == 0)
+    task_pivot<T, BS>(a, k.r, smem + L::ring_off(), cs);
+  else if constexpr (kOwnPanels<T, BS>)
+    task_panel<T, BS>(a, k.r, k.type == 1 ? k.tj : k.ti, k.type == 1, smem + L::ring_off(), cs);
   bar_compute();
   trace_stamps();
   return true;
@@ -1615,21 +1790,6 @@ __device__ __forceinline__ void publish(const Args<T>& a, const fwh::Task& k) {
     red_release_add(reinterpret_cast<unsigned*>(a.done + a.R + k.r), 1u);
 }
 
-// How a remaining-tile task relaxes: int32 over 16-bit keys when the sums of
-// its panel tiles fit (their clamp), else over 32-bit keys when those fit (1),
-// else with compare and select (0; or packed keys off).  fp32: 0, in step
-// groups; 64-bit types: 2, filtered by 16-bit bounds.
-template <typename T, int BS>
-__device__ __forceinline__ int minplus_mode(const Args<T>& a, const fwh::Task& k) {
-  if (!Num<T>::kPacked) return sizeof(T) == 8 ? 2 : 0;
-  if (!(a.packed && (k.type == 3 || k.type == kFusedTask))) return 0;
-  const int slot = k.r & 1;
-  const int ba = __ldcg(a.colB + (size_t)slot * a.slot_tiles + k.ti);
-  const int bb = __ldcg(a.rowB + (size_t)slot * a.slot_tiles + k.tj);
-  if (const int cap = h_clamp<BS>(ba, bb)) return cap;
-  return bnd_value(ba) + bnd_value(bb) < Keys<BS>::CAP ? 1 : 0;
-}
-
 // Copy the tile (k.ti, k.tj) of D into Dbuf (whole producer warp): one 2-D
 // tensor copy, or one bulk copy per valid row.
 template <typename T, int BS, int LBS>
@@ -1678,22 +1838,32 @@ __device__ __forceinline__ void issue_tile_load(const Args<T>& a, const fwh::Tas
   ++pc.d;
 }
 
-// Operand forms of a remaining tile that does not relax 16-bit keys (int32),
-// by the bounds of its panel tiles (ws_panel writes one snapshot): kFormH*: a
-// 16-bit snapshot, to be expanded to 32-bit keys (mode 1) or values (mode 0);
-// kFormK*: 32-bit keys to be decoded to values (mode 0).
+// How a remaining-tile task relaxes (mode) and the forms of its operands (kForm*).
+// int32: over 16-bit keys when the sums of its panel tiles fit (mode: their
+// clamp), else over 32-bit keys when those fit (1), else with compare and select
+// (0; or packed keys off).  Unless mode > 1 an operand kept in 16 bits, or in
+// exact 32-bit keys where values are wanted, is expanded by the compute warps.
+// The other types: 0, or 2 where tiles are filtered by 16-bit bounds.  (The two
+// bounds are loaded once, together: two loads more per task cost the producer
+// enough to slow tiles of 32-bit keys by 5 %.)
+struct TileForm {
+  int mode, dec;
+};
 template <typename T, int BS>
-__device__ __forceinline__ int key_operands(const Args<T>& a, const fwh::Task& k, int mode) {
-  if (!(Num<T>::kPacked && a.packed && (k.type == 3 || k.type == kFusedTask)) || mode > 1) return 0;
+__device__ __forceinline__ TileForm tile_form(const Args<T>& a, const fwh::Task& k) {
+  if (!Num<T>::kPacked) return {kFiltered<T, BS> ? 2 : 0, 0};
+  if (!(a.packed && (k.type == 3 || k.type == kFusedTask))) return {0, 0};
   const int slot = k.r & 1;
   const int ba = __ldcg(a.colB + (size_t)slot * a.slot_tiles + k.ti);
   const int bb = __ldcg(a.rowB + (size_t)slot * a.slot_tiles + k.tj);
+  if (const int cap = h_clamp<BS>(ba, bb)) return {cap, 0};
+  const int mode = bnd_value(ba) + bnd_value(bb) < Keys<BS>::CAP ? 1 : 0;
   int form = ((ba & kBndInf) ? kFormInfA : 0) | ((bb & kBndInf) ? kFormInfB : 0);
   if (ba & kBndH) form |= kFormHA;
   else if (mode == 0 && bnd_value(ba) < Keys<BS>::CAP) form |= kFormKA;
   if (bb & kBndH) form |= kFormHB;
   else if (mode == 0 && bnd_value(bb) < Keys<BS>::CAP) form |= kFormKB;
-  return form;
+  return {mode, form};
 }
 
 // Issue the operand copies of remaining-tile task k (whole producer warp).
@@ -1727,8 +1897,9 @@ __device__ void issue_operands(const Args<T>& a, const fwh::Task& k, int mode, i
     issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
     return;
   }
-  if constexpr (sizeof(T) == 8) return;
-  if (Num<T>::kPacked) issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
+  if constexpr (kFiltered<T, BS>) return;
+  constexpr bool kTileFirst = !std::is_same<T, float>::value;
+  if (kTileFirst) issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
   // operand chunks
   const unsigned char* srcA = (mode || (dec & kFormKA)) ? (const unsigned char*)(a.colK + toffA)
                                                        : (const unsigned char*)(a.colR + toffA);
@@ -1750,15 +1921,18 @@ __device__ void issue_operands(const Args<T>& a, const fwh::Task& k, int mode, i
       stepB = 0;
     }
   }
+  // floating types, small tiles: the predecessors of the B panel's rows as well
+  const unsigned bytesP = kPredSmem<T, BS> && a.P ? BS * BS * 4u : 0u;
   for (int c = 0; c < C::NC; ++c) {
     if (lane == 0) {
       const unsigned st = pc.chunk & 1;
       if (!pc.stop && mbar_wait(&wb->chunk_empty[st], ((pc.chunk >> 1) & 1) ^ 1, a.status,
                                 a.abort_flag, a.timeout_ns)) {
-        mbar_expect_tx(&wb->chunk_full[st], bytesA + bytesB);
+        mbar_expect_tx(&wb->chunk_full[st], bytesA + bytesB + bytesP);
         unsigned char* dst = smem + L::ring_off() + st * L::kStage;
         bulk_g2s(dst, srcA + c * stepA, bytesA, &wb->chunk_full[st]);
         bulk_g2s(dst + C::kChunkBytes, srcB + c * stepB, bytesB, &wb->chunk_full[st]);
+        if (bytesP) bulk_g2s(dst + 2 * C::kChunkBytes, a.rowP + toffB, bytesP, &wb->chunk_full[st]);
         pc.chunk_armed[st] = pc.chunk + 1;
       } else {
         pc.stop = true;
@@ -1767,7 +1941,7 @@ __device__ void issue_operands(const Args<T>& a, const fwh::Task& k, int mode, i
     ++pc.chunk;
   }
   // (fp32 reads the tile after the relaxation: its buffer may still be in use)
-  if (!Num<T>::kPacked) issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
+  if (!kTileFirst) issue_tile_load<T, BS, LBS>(a, k, smem, wb, pc, lane);
 }
 
 // Issue the operands of panel task k (whole producer warp): the tile into Dbuf,
@@ -1784,11 +1958,13 @@ __device__ void issue_panel_operands(const Args<T>& a, const fwh::Task& k, unsig
     const unsigned st = pc.chunk & 1;
     if (!pc.stop && mbar_wait(&wb->chunk_empty[st], ((pc.chunk >> 1) & 1) ^ 1, a.status,
                               a.abort_flag, a.timeout_ns)) {
-      mbar_expect_tx(&wb->chunk_full[st], (unsigned)C::kTile);
-      const void* src = a.piv + (size_t)(k.r & 1) * BS * BS;
-      if constexpr (std::is_same<T, float>::value)  // in step groups: A of a row panel, B of a column's
-        src = a.pivQ + ((size_t)(k.r & 1) * 2 + (k.type == 1 ? 0 : 1)) * BS * BS;
-      bulk_g2s(smem + L::ring_off() + st * L::kStage, src, (unsigned)C::kTile, &wb->chunk_full[st]);
+      // fp32, small column panels: the pivot's predecessors as well
+      const unsigned bytesP = kPredSmem<T, BS> && a.P && k.type == 2 ? BS * BS * 4u : 0u;
+      mbar_expect_tx(&wb->chunk_full[st], (unsigned)C::kTile + bytesP);
+      unsigned char* const dst = smem + L::ring_off() + st * L::kStage;
+      bulk_g2s(dst, a.piv + (size_t)(k.r & 1) * BS * BS, (unsigned)C::kTile, &wb->chunk_full[st]);
+      if (bytesP)
+        bulk_g2s(dst + C::kTile, a.pivP + (size_t)(k.r & 1) * BS * BS, bytesP, &wb->chunk_full[st]);
       pc.chunk_armed[st] = pc.chunk + 1;
     } else {
       pc.stop = true;
@@ -1867,43 +2043,63 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
 
   if (warp == kThreads / 32 + 1) {
     // ----------------------------------------------------------- publisher
-    for (unsigned i = 0;; ++i) {
-      const unsigned q = i % kPubDepth, ph = (i / kPubDepth) & 1;
-      bool ok = true;
-      if (lane == 0) ok = mbar_wait(&wb.pub_full[q], ph, src.status, src.abort_flag, src.timeout_ns);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      __syncwarp();
-      if (!ok) break;
-      const int t = wb.pubq[q][0];
-      const fwh::Task k{wb.pubq[q][1], wb.pubq[q][2], wb.pubq[q][3], wb.pubq[q][4]};
-      const int g = wb.pubq[q][5];
-      if (t < 0) break;
-      // tasks finish in hand-off order: the i-th completion is this task
-      if (lane == 0) ok = mbar_wait(&wb.task_done[q], ph, src.status, src.abort_flag, src.timeout_ns);
-      ok = __shfl_sync(0xffffffffu, ok, 0);
-      __syncwarp();
-      if (!ok) break;
-      if constexpr (Num<T>::kPacked) {
-        const int pst = (k.type == 1 || k.type == 2) ? wb.pst[q] : 0;
-        if (pst & kPstOn)
-          with_bs<kFixedBS, LBS>(src.bs(g), [&](auto B) {
-            store_panel<T, decltype(B)::value, LBS>(src.args(g), k, pst, smem, &wb, lane);
-            return 0;
-          });
-      }
+    // One lane waits and publishes: with the whole warp in step on every wait a
+    // publication came 0.35 us later, three times a round on the chain that
+    // bounds small solves (n = 1000, int64: 1.35 -> 1.39 ms).  The other lanes
+    // join for the copies of a 16-bit panel.
+    unsigned i = 0;
+    auto finish = [&](unsigned q, int t, const fwh::Task& k, int g) {
+      if (t != src.skip_task) publish(src.args(g), k);
+      if (uint64_t* tr = trace_slot(src.trace, src.trace_cap, src.trace_stride, t))
+        tr[5] = globaltimer();
+      mbar_arrive(&wb.pub_empty[q]);
+    };
+    for (;;) {
+      int pst = 0;
       if (lane == 0) {
-        if (t != src.skip_task) publish(src.args(g), k);
-        if (uint64_t* tr = trace_slot(src.trace, src.trace_cap, src.trace_stride, t))
-          tr[5] = globaltimer();
-        mbar_arrive(&wb.pub_empty[q]);
+        for (;; ++i) {
+          const unsigned q = i % kPubDepth, ph = (i / kPubDepth) & 1;
+          if (!mbar_wait(&wb.pub_full[q], ph, src.status, src.abort_flag, src.timeout_ns)) break;
+          const int t = wb.pubq[q][0];
+          const fwh::Task k{wb.pubq[q][1], wb.pubq[q][2], wb.pubq[q][3], wb.pubq[q][4]};
+          const int g = wb.pubq[q][5];
+          if (t < 0) break;
+          // tasks finish in hand-off order: the i-th completion is this task
+          if (!mbar_wait(&wb.task_done[q], ph, src.status, src.abort_flag, src.timeout_ns)) break;
+          if constexpr (Num<T>::kPacked) {
+            if ((k.type == 1 || k.type == 2) && (wb.pst[q] & kPstOn)) {
+              pst = wb.pst[q];
+              break;
+            }
+          }
+          finish(q, t, k, g);
+        }
       }
-      __syncwarp();
+      if constexpr (!Num<T>::kPacked) {
+        break;
+      } else {
+        pst = __shfl_sync(0xffffffffu, pst, 0);
+        i = __shfl_sync(0xffffffffu, i, 0);
+        __syncwarp();
+        if (!pst) break;
+        const unsigned q = i % kPubDepth;
+        const fwh::Task k{wb.pubq[q][1], wb.pubq[q][2], wb.pubq[q][3], wb.pubq[q][4]};
+        const int t = wb.pubq[q][0], g = wb.pubq[q][5];
+        with_bs<kFixedBS, LBS>(src.bs(g), [&](auto B) {
+          store_panel<T, decltype(B)::value, LBS>(src.args(g), k, pst, smem, &wb, lane);
+          return 0;
+        });
+        if (lane == 0) finish(q, t, k, g);
+        ++i;
+        __syncwarp();
+      }
     }
     return;
   }
 
   if (warp == kThreads / 32) {
     // ------------------------------------------------------------ producer
+    constexpr bool own_panels = kFixedBS > 0 && kOwnPanels<T, kFixedBS>;  // (batches: 32-bit types)
     const int64_t total = src.total();
     unsigned idesc = 0, ipub = 0;
     PipeCnt pc;
@@ -1912,8 +2108,9 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
       uint64_t t_claim = 0;
       if (lane == 0) {
         t_claim = globaltimer();
+        const int ab = ld_relaxed(src.abort_flag);  // (in flight together with the claim)
         const int64_t tt = atomicAdd(src.next, 1u);
-        if (tt < total && !ld_relaxed(src.abort_flag)) t = (int)tt;
+        if (tt < total && !ab) t = (int)tt;
       }
       // lane 0 decodes the task; the others take it by shuffle
       fwh::Task k{0, 0, 0, 0};
@@ -1943,12 +2140,10 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
       int bs = 0;
       if (t >= 0) {
         bs = src.bs(g);
-        mode = with_bs<kFixedBS, LBS>(bs, [&](auto B) {
-          return minplus_mode<T, decltype(B)::value>(src.args(g), k);
-        });
-        dec = with_bs<kFixedBS, LBS>(bs, [&](auto B) {
-          return key_operands<T, decltype(B)::value>(src.args(g), k, mode);
-        });
+        const TileForm form = with_bs<kFixedBS, LBS>(
+            bs, [&](auto B) { return tile_form<T, decltype(B)::value>(src.args(g), k); });
+        mode = form.mode;
+        dec = form.dec;
       }
       unsigned pq = 0;
       if (lane == 0) {
@@ -1991,15 +2186,16 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
           mbar_wait(&wb.pub_empty[pq], (((ipub - 1) / kPubDepth) & 1), src.status,
                     src.abort_flag, src.timeout_ns);
         }
-      } else if (k.type != 0) {
+      } else if (k.type != 0 && !own_panels) {
         with_bs<kFixedBS, LBS>(bs, [&](auto B) {
-          issue_panel_operands<T, decltype(B)::value, LBS>(src.args(g), k, smem, &wb, pc, lane);
+          if constexpr (!own_panels)
+            issue_panel_operands<T, decltype(B)::value, LBS>(src.args(g), k, smem, &wb, pc, lane);
           return 0;
         });
       } else {
         if (lane == 0) {
-          // a pivot task uses the shared buffer as scratch: wait until it has
-          // been published (its publication-queue slot frees up)
+          // the task uses the shared buffer as scratch: wait until it has been
+          // published (its publication-queue slot frees up)
           mbar_wait(&wb.pub_empty[pq], (((ipub - 1) / kPubDepth) & 1), src.status,
                     src.abort_flag, src.timeout_ns);
         }
@@ -2010,7 +2206,7 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
           tr[4] = globaltimer();
         }
       }
-      if (k.type == 0 || k.type == kFusedTask) fence_proxy_async();
+      if (k.type == 0 || k.type == kFusedTask || (own_panels && k.type != 3)) fence_proxy_async();
       __syncwarp();
     }
     // leave no bulk copy in flight: wait (bounded, whatever the abort flag
@@ -2058,10 +2254,14 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
   }
 }
 
-// One graph: the queue of decode_task, block size BS.
+// One graph: the queue of decode_task, block size BS.  `a` lies in shared memory:
+// as a local copy per thread (the tensor-map pointers are filled in here) its
+// lines took most of the L1 cache that 226 KB of shared memory leave, and many a
+// pointer or size that a task reads came from L2 (panels of 128: 2 to 3 K of 92 K
+// cycles).
 template <typename T, int BS>
 struct SingleSrc {
-  Args<T> a;
+  const Args<T>& a;
   unsigned* next;
   int* status;
   int* abort_flag;
@@ -2069,33 +2269,42 @@ struct SingleSrc {
   int skip_task;
   uint64_t* trace;
   int trace_cap, trace_stride;
-  __device__ SingleSrc(const Args<T>& x, const void* tmapD, const void* tmapP)
-      : a(x), next(x.ctr), status(x.status), abort_flag(x.abort_flag), timeout_ns(x.timeout_ns),
-        skip_task(x.skip_task), trace(x.trace), trace_cap(x.trace_cap),
-        trace_stride(x.trace_stride) {
-    a.tmapD = tmapD;
-    a.tmapP = tmapP;
-  }
-  __device__ int64_t total() const { return a.stage_off[a.R + 1]; }
+  int R;
+  int64_t lookahead;
+  const unsigned* stage_off;
+  mutable int stage = 0;   // of the latest task that resolve decoded
+  __device__ SingleSrc(const Args<T>& x, const Args<T>& shared)
+      : a(shared), next(x.ctr), status(x.status), abort_flag(x.abort_flag),
+        timeout_ns(x.timeout_ns), skip_task(x.skip_task), trace(x.trace),
+        trace_cap(x.trace_cap), trace_stride(x.trace_stride), R(x.R), lookahead(x.lookahead),
+        stage_off(x.stage_off) {}
+  __device__ int64_t total() const { return stage_off[R + 1]; }
   __device__ fwh::Task resolve(int64_t t, int& g) const {
     g = 0;
-    return fwh::decode_task(t, a.R, a.lookahead, a.stage_off);
+    return fwh::decode_task(t, R, lookahead, stage_off, stage);
   }
   __device__ const Args<T>& args(int) const { return a; }
   __device__ int bs(int) const { return BS; }
 };
 
-// 64-bit types: two CTAs per SM (102 registers per thread), so that the gathers
+// Filtered tiles: two CTAs per SM (102 registers per thread), so that the gathers
 // of one's exact relaxations overlap the other's work.
 template <typename T, int BS>
-__global__ void __launch_bounds__(kWsThreads, sizeof(T) == 8 ? 2 : 1)
+__global__ void __launch_bounds__(kWsThreads, kFiltered<T, BS> ? 2 : 1)
     k_persistent_ws(Args<T> a, const __grid_constant__ CUtensorMap tmD,
                     const __grid_constant__ CUtensorMap tmP, int use_tmap) {
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ WsBars wb;
   __shared__ CtaScratch cs;
   // use_tmap: bit 0 the D map, bit 1 the P map
-  const SingleSrc<T, BS> src(a, (use_tmap & 1) ? &tmD : nullptr, (use_tmap & 2) ? &tmP : nullptr);
+  __shared__ Args<T> args;
+  if (threadIdx.x == 0) {
+    args = a;
+    args.tmapD = (use_tmap & 1) ? &tmD : nullptr;
+    args.tmapP = (use_tmap & 2) ? &tmP : nullptr;
+  }
+  // (ws_engine's first barrier precedes every use)
+  const SingleSrc<T, BS> src(a, args);
   ws_engine<T, BS, BS>(src, smem, wb, cs);
 }
 
