@@ -83,7 +83,7 @@ cudaError_t run(T* D, int32_t* P, int64_t n, int64_t ld, unsigned char* base, in
   }
 
   const size_t smem = WsLayout<BS, T>::bytes();
-  auto kern = k_persistent_ws<T, BS>;
+  auto kern = persistent_kernel<T, BS>(R);
   if ((e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) !=
       cudaSuccess)
     return e;

@@ -87,7 +87,7 @@ cudaError_t launch_bs(T* D, int32_t* P, int64_t n, int64_t ld, const fwh::SolveW
       if ((e = cudaGetLastError()) != cudaSuccess) return e;
     }
   } else {
-    auto kern = k_persistent_ws<T, BS>;
+    auto kern = persistent_kernel<T, BS>(R);
     const size_t wsmem = WsLayout<BS, T>::bytes();
     const int occ = fwh::kernel_setup(reinterpret_cast<const void*>(kern), wsmem, kWsThreads);
     if (occ < 1) return cudaErrorInvalidConfiguration;

@@ -1373,9 +1373,9 @@ __device__ __noinline__ bool ws_panel_finish(const Args<T>& a, int r, int t, T* 
 // tile's own values are in Dbuf, cap is the clamp of the operands' keys.  The
 // live tile and the 16-bit snapshot are formed in the two ring stages and the
 // publisher stores them in bulk (store_panel).  The accumulators go through
-// shared memory and a short loop decodes them: decoded in registers, the
-// unrolled code of 64 entries runs once per task from a cold instruction
-// cache (8-14 K SM cycles for what the loop does in 3 K).  The results'
+// shared memory and a short loop decodes them row by row: decoded in registers,
+// with a branch and a scattered store for each of 64 entries, they took 8-14 K SM
+// cycles, the loop 3 K.  The results'
 // finite values are below cap, so the tile always has a 16-bit snapshot and
 // needs no other.
 template <typename T, int BS, int LBS, bool is_row>
@@ -1654,7 +1654,7 @@ __device__ bool compute_task(const Args<T>& a, const fwh::Task& k, int mode, int
       ok = ws_minplus_f<T, BS, LBS>(a, k, smem, wb, pc, tr);
     } else {
       const TileCtx<T> ctx{a.D, a.P, a.n, a.ld, k.r, a.status, a.abort_flag, a.timeout_ns};
-      ok = ws_minplus<T, BS, LBS, false, false>(ctx, k.ti, k.tj, 0, smem, wb, pc, tr);
+      ok = ws_minplus_body<T, BS, LBS, false, false>(ctx, k.ti, k.tj, 0, smem, wb, pc, tr);
     }
     if (!ok || k.type == 3) return ok;
     // fused: the tile's stores precede the pivot's loads of it (same CTA),
@@ -2287,10 +2287,8 @@ struct SingleSrc {
   __device__ int bs(int) const { return BS; }
 };
 
-// Filtered tiles: two CTAs per SM (102 registers per thread), so that the gathers
-// of one's exact relaxations overlap the other's work.
-template <typename T, int BS>
-__global__ void __launch_bounds__(kWsThreads, kFiltered<T, BS> ? 2 : 1)
+template <typename T, int BS, int kCtas>
+__global__ void __launch_bounds__(kWsThreads, kCtas)
     k_persistent_ws(Args<T> a, const __grid_constant__ CUtensorMap tmD,
                     const __grid_constant__ CUtensorMap tmP, int use_tmap) {
   extern __shared__ __align__(128) unsigned char smem[];
@@ -2306,6 +2304,23 @@ __global__ void __launch_bounds__(kWsThreads, kFiltered<T, BS> ? 2 : 1)
   // (ws_engine's first barrier precedes every use)
   const SingleSrc<T, BS> src(a, args);
   ws_engine<T, BS, BS>(src, smem, wb, cs);
+}
+
+// The kernel for R x R tiles, by CTAs per SM.  Filtered fp64: two (102 registers
+// per thread), so that the gathers of one's exact relaxations overlap the other's
+// work.  Tiles of 64 with 32-bit elements: a tile is done in 2.7 us (int32, 16-bit
+// keys) to 7 us (fp32), in which a lone CTA waits for its operands half of the
+// time; two overlap that, but also share the SM with the tasks that the chain of
+// pivots waits for.  From 12 tiles per SM and round on the first counts more (one /
+// two CTAs per SM, int32 R = 36 1.34 / 1.42 ms, R = 41 1.83 / 1.77, R = 47 2.62 /
+// 2.22; weights to 3e5, R = 41 1.91 / 1.92, R = 47 2.75 / 2.60; fp32 R = 36 2.15 /
+// 2.17, R = 41 3.04 / 2.79, R = 47 4.53 / 4.26).  The kernel for one CTA keeps its
+// 168 registers (at 102 it is 2 % slower: n = 1000 0.60 -> 0.61 ms).
+template <typename T, int BS>
+auto persistent_kernel(int R) {
+  if constexpr (BS == 64 && sizeof(T) == 4)
+    if ((int64_t)R * R >= 12 * (int64_t)fwh::num_sms()) return k_persistent_ws<T, BS, 2>;
+  return k_persistent_ws<T, BS, kFiltered<T, BS> ? 2 : 1>;
 }
 
 }  // namespace fwk

@@ -64,3 +64,16 @@ def test_negative_cycle_across_tiles(dtype):
         gpu_solve(W, bs=64)
     assert e.value.code == 4
     gpu_solve(_weights(dtype, 90, "uniform", seed=5), bs=64)  # the status was cleared
+
+
+@pytest.mark.parametrize("dtype", [np.int32, np.float32])
+@pytest.mark.parametrize("n", [64 * 42, 64 * 42 + 1, 64 * 44 - 3])
+def test_two_ctas_per_sm(dtype, n):
+    """Blocks of 64 with 32-bit elements, around the size from which two CTAs
+    share an SM."""
+    W = _weights(np.float32, n, "small", seed=n)
+    if dtype is np.int32:
+        W = np.where(np.isinf(W), 1 << 29, W).astype(np.int32)
+    D, P = gpu_solve(W, bs=64, driver=PERSISTENT)
+    Dr, Pr = gpu_solve(W, bs=64, driver=PHASED)
+    assert D.tobytes() == Dr.tobytes() and np.array_equal(P, Pr)
