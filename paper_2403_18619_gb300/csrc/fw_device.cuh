@@ -519,7 +519,7 @@ struct Args {
   int32_t* rowP;        // [2][tiles][BS*BS] predecessors of the row panel tiles
   int32_t* rowB;
   // 16-bit key snapshots of the panel tiles (int32; KeysH, put_h): [2][tiles][BS*BS/2]
-  // (64-bit types: 16-bit lower bounds in the same layout, fw_filter.cuh)
+  // (fp64: 16-bit lower bounds in the same layout, fw_filter.cuh)
   uint32_t* colH;
   uint32_t* rowH;
   int* qexp;            // [R] exponent of each round's bounds (fp64; set by its pivot)

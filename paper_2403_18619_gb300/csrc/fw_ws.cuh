@@ -367,7 +367,9 @@ __device__ __forceinline__ void turn_pass(int g) {
 // Remaining-tile task over 16-bit packed keys (int32; cap: their clamp).  The
 // accumulators hold the operands' sums only; the tile's own values are read
 // from Dbuf afterwards, so that their copy has the whole relaxation to arrive
-// and nothing converts them to keys.
+// and nothing converts them to keys.  Bound by the ALU pipe (two relaxations per
+// DPX instruction, 122 per SM clock), which the turns keep to the relaxation:
+// n = 16384 265 ms over 32-bit keys, 174 ms.
 template <typename T, int BS, int LBS>
 __device__ __noinline__ bool ws_minplus_h(const Args<T>& a, const fwh::Task& k, int cap,
                                           unsigned char* smem, WsBars* wb, PipeCnt& pc,
@@ -467,10 +469,13 @@ __device__ __forceinline__ QuadTask quad_task(const Args<float>& a, int ti, int 
   return f;
 }
 
-// Remaining-tile task of fp32.  With predecessors the groups of warps relax in
-// turns, each with the pipes to itself while the other finds the steps of what
-// it improved (n = 8192: 78 ms, 83 without turns); distances alone leave little
-// to do afterwards (n = 5000: 10.5 ms without turns, 11.9 with).
+// Remaining-tile task of fp32, bound by issue slots (eight instructions per four
+// relaxations).  Tiles of 128 with predecessors are relaxed in turns, each group of
+// warps with the pipes to itself while the other finds the steps of what it
+// improved (n = 8192: 78 ms, 83 without turns; 73 since distances leave in
+// vectors, 98 with an argmin by step); distances alone leave little to do
+// afterwards (n = 5000: 10.5 ms without turns, 11.9 with), and small tiles wait on
+// a chain, which turns lengthen (a tile of 64: 17 K SM cycles, 13.4 K without).
 template <int BS, int LBS>
 __device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task& k,
                                           unsigned char* smem, WsBars* wb, PipeCnt& pc,
@@ -769,9 +774,10 @@ __device__ __forceinline__ FilterTask<T> filter_task(const Args<T>& a, int r, in
   return f;
 }
 
-// Remaining-tile task of fp64 (BS = 64): the 16-bit pass
-// in turns, then the exact relaxation of the entries that may improve while
-// the other group of warps has its turn.
+// Remaining-tile task of fp64 (BS = 64): the 16-bit pass in turns, then the exact
+// relaxation of the entries that may improve while the other group of warps has
+// its turn.  The first rounds are bound by those relaxations, the later ones by the
+// 16-bit pass (20 K SM cycles per tile, exact 160 K): n = 4096 133 -> 27 ms.
 template <typename T, int BS, int LBS>
 __device__ __noinline__ bool ws_minplus_f(const Args<T>& a, const fwh::Task& k, unsigned char* smem,
                                           WsBars* wb, PipeCnt& pc, uint64_t* tr) {
@@ -1844,8 +1850,8 @@ __device__ __forceinline__ void issue_tile_load(const Args<T>& a, const fwh::Tas
 // (0; or packed keys off).  Unless mode > 1 an operand kept in 16 bits, or in
 // exact 32-bit keys where values are wanted, is expanded by the compute warps.
 // The other types: 0, or 2 where tiles are filtered by 16-bit bounds.  (The two
-// bounds are loaded once, together: two loads more per task cost the producer
-// enough to slow tiles of 32-bit keys by 5 %.)
+// bounds are loaded once, together: a second round trip to L2 would lie on the
+// producer's serial path, which bounds small tiles.)
 struct TileForm {
   int mode, dec;
 };

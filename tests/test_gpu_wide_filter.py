@@ -1,5 +1,5 @@
 """GPU tests (-m gpu): the persistent driver's kernels of fp32 (steps in groups
-of four), fp64 and int64 (filtered by 16-bit bounds) give, bit for bit, the
+of four), fp64 (blocks of 64 filtered by 16-bit bounds) and int64 give, bit for bit, the
 distances and predecessors of the phased driver's kernels, which relax every
 step of every entry in order: at tile edges, with ties, with missing edges, over
 wide ranges of magnitude (bounds clamped, or zero), and distances alone."""
