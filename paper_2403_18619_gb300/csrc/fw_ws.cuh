@@ -125,26 +125,24 @@ struct WsBars {
 // holds the 16-bit snapshot), and whether the tile is whole and stored so.
 constexpr int kPstOn = 1, kPstStage = 2, kPstTile = 4;
 
-// Bounded wait on an mbarrier phase; false (and the timeout status) on expiry.
-// With poll_abort, a wait that has already lasted over a millisecond (normal
-// waits take microseconds) also gives up, without recording anything, once
-// another CTA has raised the abort flag, so that one failure does not make
-// every pending wait of every CTA run out its own limit in turn.  Polling the
-// flag from the start cost the compute warps' operand waits about 1 % of the
-// n = 32768 solve.
-constexpr uint64_t kAbortPollAfterNs = 1000000;
+// Wait on an mbarrier phase of this CTA.  Such a phase ends by the CTA's own
+// progress: a descriptor that the producer hands out (the last one says stop), a
+// copy that it issues after the task's inputs from other CTAs are there, a buffer
+// that the warps leave.  Only the producer waits for other CTAs (wait_ge), and only
+// there the solve's limit and its abort flag count: the producer alone decides that
+// a solve ends early, and every warp learns of it by the same descriptor.  (With a
+// limit here, warps would give up one by one, and those that did not would be left
+// at a barrier: a turn, or the barriers of pivots and panels.)
+// False, with the timeout status, only if the phase is still open kLostNs after
+// the longest wait of the producer: a copy was lost.
+constexpr uint64_t kLostNs = 10000000000ull;
 __device__ __forceinline__ bool mbar_wait(uint64_t* bar, unsigned parity, int* status,
-                                          int* abort_flag, int64_t timeout_ns,
-                                          bool poll_abort = true) {
+                                          int* abort_flag, int64_t timeout_ns) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint64_t t0 = globaltimer();
-  for (int64_t it = 0; it < ((int64_t)1 << 26); ++it) {
+  for (int64_t it = 0; it < ((int64_t)1 << 30); ++it) {
     if (mbar_try_wait_sleep(bar, parity, 20000u)) return true;
-    if ((it & 15) == 15) {
-      const uint64_t waited = globaltimer() - t0;
-      if (waited > (uint64_t)timeout_ns) break;
-      if (poll_abort && waited > kAbortPollAfterNs && ld_relaxed(abort_flag)) return false;
-    }
+    if ((it & 15) == 15 && globaltimer() - t0 > (uint64_t)timeout_ns + kLostNs) break;
   }
   atomicOr(status, kStTimeout);
   atomicExch(abort_flag, 1);
@@ -521,7 +519,7 @@ __device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task&
     if (!kHold && lane == 0) mbar_arrive(&wb->chunk_empty[st]);
     ++pc.chunk;
   }
-  if (kTurns && a.P) turn_pass(group ^ 1);  // (also when a wait has given up: the other group must not wait for it)
+  if (kTurns && a.P) turn_pass(group ^ 1);
   if (!ok) return false;
   const long long t_b = tr ? clock64() : 0;
   if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns)) return false;
@@ -2215,16 +2213,15 @@ __device__ void ws_engine(const Src& src, unsigned char* smem, WsBars& wb, CtaSc
       if (k.type == 0 || k.type == kFusedTask || (own_panels && k.type != 3)) fence_proxy_async();
       __syncwarp();
     }
-    // leave no bulk copy in flight: wait (bounded, whatever the abort flag
-    // says) for the last phase armed with a copy on every full barrier
+    // leave no bulk copy in flight: wait for the last phase armed with a copy on
+    // every full barrier
     if (lane == 0) {
       if (pc.d_armed)
-        mbar_wait(&wb.d_full, (pc.d_armed - 1) & 1, src.status, src.abort_flag, src.timeout_ns,
-                  false);
+        mbar_wait(&wb.d_full, (pc.d_armed - 1) & 1, src.status, src.abort_flag, src.timeout_ns);
       for (int st = 0; st < 2; ++st)
         if (pc.chunk_armed[st])
           mbar_wait(&wb.chunk_full[st], ((pc.chunk_armed[st] - 1) >> 1) & 1, src.status,
-                    src.abort_flag, src.timeout_ns, false);
+                    src.abort_flag, src.timeout_ns);
     }
     return;
   }
