@@ -349,9 +349,9 @@ __device__ __forceinline__ T vmin(T a, T b) {
 
 // Whether the remaining tiles and panels are filtered by 16-bit bounds
 // (fw_filter.cuh): fp64 in blocks of 64.  Its exact relaxation of a tile takes
-// 160 K SM cycles there, the filtered one 400 K in the first round, where every
-// entry improves, and 20-60 K later (n = 700: 2.86 -> 2.40 ms, n = 4096: 133 ->
-// 28 ms).  At BS = 32 (n <= 512) a tile takes 19 K cycles and the rounds are
+// 160 K SM cycles there, the filtered one 20-60 K after the first rounds (n = 700:
+// 2.87 -> 2.01 ms, n = 4096: 133 -> 26.3 ms); tiles whose bounds say little are
+// relaxed exactly after all.  At BS = 32 (n <= 512) a tile takes 19 K cycles and the rounds are
 // bound by their chain, which filtered panels lengthen (n = 400: 0.59 -> 0.68
 // ms).  int64 relaxes a tile in 36 K cycles; filtered, n = 1000 went from 1.34 to
 // 2.13 ms and n = 3000 only from 12.9 to 11.8.
@@ -411,13 +411,17 @@ struct Quant<double> {
   static constexpr int kMinExp = -100, kMaxExp = 100;
 };
 
-// The round's exponent from the leading bit of the closed pivot's largest
-// finite entry, which lands in [4096, 8192): the entries that matter, sums that
-// undercut an entry, lie below.  `prev`: the exponent to keep when the pivot has no such entry.
+// The round's exponent from the leading bit of a typical entry of the closed pivot
+// (pivot_exponent), which lands in [2^kTypicalBit, 2^(kTypicalBit + 1)): the sums that
+// undercut an entry are of its size or below, and the few entries eight times
+// larger than it or more saturate.  (Scaled by the largest entry, one vertex far
+// from the others in a block of 64 made every ordinary bound 0: n = 4096 134 ms,
+// now 71.  Bits 9, 10 and 11: a grid of n = 4096 19.2, 19.2 and 43.5 ms, its
+// distances spread over the scale; uniform n = 4096 26.6, 26.2 and 26.1.)
+constexpr int kTypicalBit = 10;
 template <typename T>
-__device__ __forceinline__ int q_exponent(int lead, int prev) {
-  if (lead == kNoLead) return prev;
-  return min(max(12 - lead, Quant<T>::kMinExp), Quant<T>::kMaxExp);
+__device__ __forceinline__ int q_exponent(int lead) {
+  return min(max(kTypicalBit - lead, Quant<T>::kMinExp), Quant<T>::kMaxExp);
 }
 
 // Raw vector of NB bytes and G elements viewed as one value (8-byte elements).
@@ -726,13 +730,14 @@ __device__ __forceinline__ int32_t resolve_pred(int32_t p, const int32_t* P, int
   return p;
 }
 
-// CTA-wide maxima of N ints (every thread gets the results).
-template <int N>
-__device__ __forceinline__ void block_max(int (&v)[N], CtaScratch* cs) {
+// CTA-wide maxima (kSum: sums) of N ints (every thread gets the results).
+template <bool kSum, int N>
+__device__ __forceinline__ void block_reduce(int (&v)[N], CtaScratch* cs) {
   static_assert(N <= 4, "CtaScratch::red");
   const int w = threadIdx.x >> 5;
 #pragma unroll
-  for (int i = 0; i < N; ++i) v[i] = __reduce_max_sync(0xffffffffu, v[i]);
+  for (int i = 0; i < N; ++i)
+    v[i] = kSum ? __reduce_add_sync(0xffffffffu, v[i]) : __reduce_max_sync(0xffffffffu, v[i]);
   bar_compute();
   if ((threadIdx.x & 31) == 0) {
 #pragma unroll
@@ -743,8 +748,13 @@ __device__ __forceinline__ void block_max(int (&v)[N], CtaScratch* cs) {
   for (int i = 0; i < N; ++i) {
     v[i] = cs->red[i][0];
 #pragma unroll
-    for (int k = 1; k < kThreads / 32; ++k) v[i] = max(v[i], cs->red[i][k]);
+    for (int k = 1; k < kThreads / 32; ++k)
+      v[i] = kSum ? v[i] + cs->red[i][k] : max(v[i], cs->red[i][k]);
   }
+}
+template <int N>
+__device__ __forceinline__ void block_max(int (&v)[N], CtaScratch* cs) {
+  block_reduce<false>(v, cs);
 }
 __device__ __forceinline__ void block_max2(int& a, int& b, CtaScratch* cs) {
   int v[2] = {a, b};
@@ -1374,6 +1384,35 @@ __device__ __forceinline__ void closure_steps(T (&d)[Geo<BS>::TM][Geo<BS>::TM],
   }
 }
 
+// Exponent of a round's 16-bit bounds (fw_filter.cuh) from its closed pivot: the
+// mean leading bit of the positive finite entries at or below their mean leading
+// bit.  (The first mean alone moves with a large finite weight in half of the
+// entries.)  `prev`: the one to keep when there is no such entry.
+template <typename T, int BS>
+__device__ __forceinline__ int pivot_exponent(const T (&d)[Geo<BS>::TM][Geo<BS>::TM],
+                                              CtaScratch* cs, int prev) {
+  constexpr int TM = Geo<BS>::TM;
+  int top = 1 << 20, mean = kNoLead;
+#pragma unroll 1
+  for (int pass = 0; pass < 2; ++pass) {
+    int sum[2] = {0, 0};  // leading bits, and how many
+#pragma unroll
+    for (int m = 0; m < TM; ++m)
+#pragma unroll
+      for (int nn = 0; nn < TM; ++nn) {
+        const int lead = Quant<T>::lead(d[m][nn]);
+        const bool in = lead != kNoLead && lead <= top;
+        sum[0] += in ? lead : 0;
+        sum[1] += in ? 1 : 0;
+      }
+    block_reduce<true>(sum, cs);
+    if (sum[1] == 0) return prev;
+    // (rounded up: some entry is at or below it)
+    top = mean = sum[0] >= 0 ? (sum[0] + sum[1] - 1) / sum[1] : -(-sum[0] / sum[1]);
+  }
+  return q_exponent<T>(mean);
+}
+
 // Eager pivot: compare and select per relaxation (fp32, 64-bit types, large
 // int32 entries).
 template <typename T, int BS>
@@ -1396,14 +1435,8 @@ __device__ __noinline__ void pivot_eager(const Args<T>& a, int r, void* smem_raw
   closure_steps<T, BS>(d, p, smem_raw);
   stamp(2);
   if constexpr (kFiltered<T, BS>) {
-    // the exponent of the round's 16-bit bounds (fw_filter.cuh)
-    int lead[1] = {kNoLead};
-#pragma unroll
-    for (int mm = 0; mm < TM; ++mm)
-#pragma unroll
-      for (int nn = 0; nn < TM; ++nn) lead[0] = max(lead[0], Quant<T>::lead(d[mm][nn]));
-    block_max(lead, cs);
-    if (tid == 0) a.qexp[r] = q_exponent<T>(lead[0], r ? __ldcg(a.qexp + r - 1) : 0);
+    const int e = pivot_exponent<T, BS>(d, cs, r ? __ldcg(a.qexp + r - 1) : 0);
+    if (tid == 0) a.qexp[r] = e;
   }
   stamp(3);
   pivot_store_dist<T, BS>(a, r, d, tx, ty);

@@ -177,6 +177,7 @@ struct PipeCnt {
   unsigned d = 0, chunk = 0;
   unsigned d_armed = 0, chunk_armed[2] = {0, 0};
   bool stop = false;
+  int exact = -2;  // (filtered fp64) skip_filter
 };
 
 // ------------------------------------------------------------ compute side ----
@@ -772,17 +773,77 @@ __device__ __forceinline__ FilterTask<T> filter_task(const Args<T>& a, int r, in
   return f;
 }
 
+// A remaining-tile task's FilterTask; its operands' bounds are in the ring stage st.
+template <typename T, int BS, int LBS>
+__device__ __forceinline__ FilterTask<T> tile_filter(const Args<T>& a, const fwh::Task& k,
+                                                     unsigned char* smem, unsigned st) {
+  using L = WsLayout<LBS, T>;
+  FilterTask<T> f = filter_task<T, BS>(a, k.r, k.ti, k.tj);
+  const size_t ta = (size_t)(k.r & 1) * a.slot_tiles + k.ti, tb = (size_t)(k.r & 1) * a.slot_tiles + k.tj;
+  f.A = a.colR + ta * BS * BS;
+  f.B = a.rowR + tb * BS * BS;
+  f.old = reinterpret_cast<const T*>(smem + L::d_off());
+  f.Ah = reinterpret_cast<const uint32_t*>(smem + L::ring_off() + st * L::kStage);
+  f.Bh = f.Ah + KeysH<BS>::kTileWords;
+  if (!ViaPred<T>::kOn) f.Psrc = a.rowP + tb * BS * BS;
+  f.neg = __ldcg(a.colB + ta) | __ldcg(a.rowB + tb);
+  return f;
+}
+
+// Releases the buffers of a remaining-tile task.  Whole warp.
+__device__ __forceinline__ void leave_tile_f(WsBars* wb, PipeCnt& pc) {
+  __syncwarp();
+  if ((threadIdx.x & 31) == 0) {
+    mbar_arrive(&wb->chunk_empty[pc.chunk & 1]);
+    mbar_arrive(&wb->d_empty);
+  }
+  ++pc.chunk;
+  ++pc.d;
+}
+
+// Remaining-tile task of fp64 (BS = 64) over every step of every entry, after the
+// filter's turn (ws_minplus_f) or, with kSkip, without it: the whole task.  Out of
+// line and not called from ws_minplus_f, whose tiles paid 3 to 5 % for the call.
+template <typename T, int BS, int LBS, bool kSkip>
+__device__ __noinline__ bool ws_exact_f(const Args<T>& a, const fwh::Task& k, unsigned char* smem,
+                                        WsBars* wb, PipeCnt& pc, uint64_t* tr) {
+  const unsigned st = pc.chunk & 1;
+  const long long t_a = tr ? clock64() : 0;
+  if (kSkip) {
+    const int group = (int)threadIdx.x >> 7;
+    if (!mbar_wait(&wb->chunk_full[st], (pc.chunk >> 1) & 1, a.status, a.abort_flag, a.timeout_ns))
+      return false;
+    const long long cw = tr ? clock64() - t_a : 0;
+    turn_wait(group);
+    turn_pass(group ^ 1);
+    const long long t_b = tr ? clock64() : 0;
+    if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns)) return false;
+    if (tr) {
+      tr[7] = cyc20(clock64() - t_b) | (cyc20(cw) << 20);
+      tr[8] = 0;
+    }
+  }
+  int tx, ty;
+  h_thread(tx, ty);
+  relax_exact<T, BS, true>(tile_filter<T, BS, LBS>(a, k, smem, st), tx, ty);
+  leave_tile_f(wb, pc);
+  if (tr) {  // (the cycles of the relaxation come on top of the filter's)
+    const uint64_t t = (uint64_t)(clock64() - t_a);
+    tr[8] += t | t << 32;
+  }
+  return true;
+}
+
 // Remaining-tile task of fp64 (BS = 64): the 16-bit pass in turns, then the exact
 // relaxation of the entries that may improve while the other group of warps has
 // its turn.  The first rounds are bound by those relaxations, the later ones by the
 // 16-bit pass (20 K SM cycles per tile, exact 160 K): n = 4096 133 -> 27 ms.
 template <typename T, int BS, int LBS>
 __device__ __noinline__ bool ws_minplus_f(const Args<T>& a, const fwh::Task& k, unsigned char* smem,
-                                          WsBars* wb, PipeCnt& pc, uint64_t* tr) {
+                                          WsBars* wb, PipeCnt& pc, uint64_t* tr, bool& exact) {
   using H = KeysH<BS>;
   using L = WsLayout<LBS, T>;
   constexpr int TM = Geo<BS>::TM;
-  const int lane = threadIdx.x & 31;
   int tx, ty;
   h_thread(tx, ty);
   const unsigned st = pc.chunk & 1;
@@ -806,24 +867,11 @@ __device__ __noinline__ bool ws_minplus_f(const Args<T>& a, const fwh::Task& k, 
     tr[7] = cyc20(clock64() - t_b) | (cyc20(cw) << 20);
     tr[8] = (uint64_t)(t_b - t_a);
   }
-  FilterTask<T> f = filter_task<T, BS>(a, k.r, k.ti, k.tj);
-  const size_t ta = (size_t)(k.r & 1) * a.slot_tiles + k.ti, tb = (size_t)(k.r & 1) * a.slot_tiles + k.tj;
-  f.A = a.colR + ta * BS * BS;
-  f.B = a.rowR + tb * BS * BS;
-  f.old = reinterpret_cast<const T*>(smem + L::d_off());
-  f.Ah = As;
-  f.Bh = As + H::kTileWords;
-  if (!ViaPred<T>::kOn) f.Psrc = a.rowP + tb * BS * BS;
-  f.neg = __ldcg(a.colB + ta) | __ldcg(a.rowB + tb);
-  refine_tile<T, BS, true>(f, acc, tx, ty,
-                     reinterpret_cast<uint32_t*>(smem + L::scr_off() + (threadIdx.x >> 5) * L::kScrWarp));
-  __syncwarp();
-  if (lane == 0) {
-    mbar_arrive(&wb->chunk_empty[st]);
-    mbar_arrive(&wb->d_empty);
-  }
-  ++pc.chunk;
-  ++pc.d;
+  const FilterTask<T> f = tile_filter<T, BS, LBS>(a, k, smem, st);
+  exact = !refine_tile<T, BS, true>(f, acc, tx, ty,
+                                    reinterpret_cast<uint32_t*>(smem + L::scr_off() +
+                                                                (threadIdx.x >> 5) * L::kScrWarp));
+  if (!exact) leave_tile_f(wb, pc);
   if (tr) tr[8] |= (uint64_t)(clock64() - t_a) << 32;
   return true;
 }
@@ -858,6 +906,13 @@ __device__ __forceinline__ int quantize_tile(uint32_t* H, const QScale& q, Src&&
     else *u = word[0];
   }
   return neg;
+}
+
+// (out of line, as ws_exact_f)
+template <typename T, int BS>
+__device__ __noinline__ void panel_exact(const FilterTask<T>& f, int tx, int ty) {
+  relax_exact<T, BS, false>(f, tx, ty);
+  __syncwarp();
 }
 
 // Panel task of round r of fp64 (BS = 64): Dbuf holds the tile's own values,
@@ -915,8 +970,10 @@ __device__ __noinline__ bool ws_panel_f(const Args<T>& a, const fwh::Task& k, un
   f.Bh = Bh;
   if (!ViaPred<T>::kOn) f.Psrc = is_row ? snapP : a.pivP + (size_t)(r & 1) * BS * BS;
   f.neg = neg[0] != 0;
-  refine_tile<T, BS, false>(f, acc, tx, ty,
-                     reinterpret_cast<uint32_t*>(smem + L::scr_off() + (threadIdx.x >> 5) * L::kScrWarp));
+  if (!refine_tile<T, BS, false>(f, acc, tx, ty,
+                                 reinterpret_cast<uint32_t*>(smem + L::scr_off() +
+                                                             (threadIdx.x >> 5) * L::kScrWarp)))
+    panel_exact<T, BS>(f, tx, ty);
   fence_proxy_async_shared();  // generic writes before the stage's next TMA fill
   bar_compute();  // the relaxed tile is in the matrix, the operands are free
   stamp(2);
@@ -1655,7 +1712,16 @@ __device__ bool compute_task(const Args<T>& a, const fwh::Task& k, int mode, int
     } else if constexpr (sizeof(T) == 4) {
       ok = ws_minplus_q<BS, LBS>(a, k, smem, wb, pc, tr);
     } else if constexpr (kFiltered<T, BS>) {
-      ok = ws_minplus_f<T, BS, LBS>(a, k, smem, wb, pc, tr);
+      if (skip_filter(pc.exact, k.r, k.ti, k.tj)) {
+        ok = ws_exact_f<T, BS, LBS, true>(a, k, smem, wb, pc, tr);
+      } else {
+        bool exact = false;
+        ok = ws_minplus_f<T, BS, LBS>(a, k, smem, wb, pc, tr, exact);
+        if (exact) {
+          pc.exact = k.r;
+          ok = ws_exact_f<T, BS, LBS, false>(a, k, smem, wb, pc, tr);
+        }
+      }
     } else {
       const TileCtx<T> ctx{a.D, a.P, a.n, a.ld, k.r, a.status, a.abort_flag, a.timeout_ns};
       ok = ws_minplus_body<T, BS, LBS, false, false>(ctx, k.ti, k.tj, 0, smem, wb, pc, tr);
@@ -2309,9 +2375,14 @@ __global__ void __launch_bounds__(kWsThreads, kCtas)
   ws_engine<T, BS, BS>(src, smem, wb, cs);
 }
 
-// The kernel for R x R tiles, by CTAs per SM.  Filtered fp64: two (102 registers
+// The kernel for R x R tiles, by CTAs per SM.  Filtered fp64: two (96 registers
 // per thread), so that the gathers of one's exact relaxations overlap the other's
-// work.  Tiles of 64 with 32-bit elements: a tile is done in 2.7 us (int32, 16-bit
+// work, from five tiles per SM and round on.  With fewer, tiles and the chain of
+// pivots would share an SM's narrow FP64 pipe while other SMs are idle (two / one
+// CTA per SM, uniform n = 700 2.47 / 2.02 ms, n = 1100 3.58 / 3.02, n = 1650 5.12 /
+// 4.57, n = 1800 5.70 / 5.33; a far vertex in each block n = 900 4.1 / 3.7, n = 1350
+// 6.1 / 5.7, n = 1650 7.6 / 9.2, n = 1800 8.6 / 11.7).
+// Tiles of 64 with 32-bit elements: a tile is done in 2.7 us (int32, 16-bit
 // keys) to 7 us (fp32), in which a lone CTA waits for its operands half of the
 // time; two overlap that, but also share the SM with the tasks that the chain of
 // pivots waits for.  From 12 tiles per SM and round on the first counts more (one /
@@ -2323,7 +2394,9 @@ template <typename T, int BS>
 auto persistent_kernel(int R) {
   if constexpr (BS == 64 && sizeof(T) == 4)
     if ((int64_t)R * R >= 12 * (int64_t)fwh::num_sms()) return k_persistent_ws<T, BS, 2>;
-  return k_persistent_ws<T, BS, kFiltered<T, BS> ? 2 : 1>;
+  if constexpr (kFiltered<T, BS>)
+    if ((int64_t)R * R > 5 * (int64_t)fwh::num_sms()) return k_persistent_ws<T, BS, 2>;
+  return k_persistent_ws<T, BS, 1>;
 }
 
 }  // namespace fwk
