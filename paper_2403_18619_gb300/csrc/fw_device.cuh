@@ -774,10 +774,38 @@ __device__ __forceinline__ void core_packed(const uint32_t* __restrict__ As,
                                             int ty) {
   using Gm = Geo<BS>;
   constexpr int G = Gm::G, TM = Gm::TM;
-  // Unrolled 8 steps: measured at n = 32768 (2.18 / 2.12 / 2.08 / 2.09 / 2.22 / 2.23 s
-  // per solve for 2 / 4 / 8 / 16 / 32 / 64): the loop's address and branch
-  // instructions share the ALU pipe with the DPX relaxations; beyond 8 the
-  // loop body outgrows the instruction cache.
+  if constexpr (BS == 128) {
+    // Eight steps per pass of the loop, a step's operands loaded during the one
+    // before: nothing else hides the loads of a pass's first step, and whether the
+    // compiler moves them up varied with the code around the loop (n = 8000, weights
+    // to 1e6: 33.1 ms, 33.8 when it did not, 33.4 so; 4 steps per pass 33.6, 16 35.4).
+    uint32_t a[2][TM], b[2][TM];
+    auto load = [&](int h, int kk) {
+#pragma unroll
+      for (int g = 0; g < Gm::NG; ++g) {
+        uint32_t ta[G], tb[G];
+        vload_s<G>(ta, As + kk * BS + g * Gm::SPAN + ty * G);
+        vload_s<G>(tb, Bs + kk * BS + g * Gm::SPAN + tx * G);
+#pragma unroll
+        for (int e = 0; e < G; ++e) { a[h][g * G + e] = ta[e]; b[h][g * G + e] = tb[e]; }
+      }
+    };
+    load(0, 0);
+#pragma unroll 4
+    for (int kk = 0; kk < K; kk += 2) {
+#pragma unroll
+      for (int h = 0; h < 2; ++h) {
+        load(h ^ 1, kk + h + 1 < K ? kk + h + 1 : K - 1);
+#pragma unroll
+        for (int m = 0; m < TM; ++m)
+#pragma unroll
+          for (int nn = 0; nn < TM; ++nn)
+            acc[m][nn] = __viaddmin_u32(a[h][m], b[h][nn], acc[m][nn]);
+      }
+    }
+    return;
+  }
+  // (smaller blocks: the loop as it is, n = 3000 2.65 ms, 2.70 with operands ahead)
 #pragma unroll 8
   for (int kk = 0; kk < K; ++kk) {
     uint32_t a[TM], b[TM];
