@@ -269,10 +269,10 @@ struct KeysH {
   static constexpr int kTileWords = BS * BS / 2;
   static_assert((1 << KB) == BS && 2 * (kCapI << KB) + BS <= (1 << 16), "16-bit keys");
 };
-// What a panel tile publishes beside its snapshot: the bound of its finite
-// entries, whether an entry is INF, and whether the snapshot is of 16-bit keys.
-constexpr int kBndInf = 1 << 30, kBndH = 1 << 29;
-__host__ __device__ constexpr int bnd_value(int b) { return b & (kBndH - 1); }
+// What a panel tile publishes beside its snapshots: the bound of its finite
+// entries, whether an entry is INF, and whether there are 16-bit and 32-bit keys.
+constexpr int kBndInf = 1 << 30, kBndH = 1 << 29, kBndK = 1 << 28;
+__host__ __device__ constexpr int bnd_value(int b) { return b & (kBndK - 1); }
 // Clamp of the 16-bit keys of two tiles with these bounds; 0 when they cannot
 // hold their sums (or a snapshot is of another kind).
 template <int BS>

@@ -1316,11 +1316,13 @@ __device__ __noinline__ bool ws_panel_finish(const Args<T>& a, int r, int t, T* 
     has_inf = b.inf();
   }
   block_max2(nb, has_inf, cs);
-  // one snapshot: 16-bit keys where the bound allows them, else 32-bit keys,
-  // which are exact while every finite value is below CAP; beyond that the raw
-  // values as well, and without packed keys the raw values only
+  // snapshots: 32-bit keys, which are exact while every finite value is below CAP;
+  // beyond that the raw values as well, and without packed keys the raw values
+  // only.  16-bit keys too where the bound allows them (16-bit keys alone, expanded
+  // where the other operand of a tile has none: a grid of n = 8100 34.2 ms, 31.8
+  // with both; n = 8000 of degree 8, weights to 100, 35.1 and 34.5).
   const bool hok = a.packed && h_tile_ok<BS>(nb | has_inf);
-  const bool keys = a.packed && !hok;
+  const bool keys = a.packed != 0;
   const bool raw = !a.packed || nb >= K::CAP;
   const int slot = r & 1;
   const size_t tile_off = ((size_t)slot * a.slot_tiles + t) * BS * BS;
@@ -1424,7 +1426,7 @@ __device__ __noinline__ bool ws_panel_finish(const Args<T>& a, int r, int t, T* 
     else
       put_h<BS, true>(snapH, tx, ty, [&](int k, int q) { return key16(q, k); });
   }
-  if (tid == 0) *bnd = nb | has_inf | (hok ? kBndH : 0);
+  if (tid == 0) *bnd = nb | has_inf | (hok ? kBndH : 0) | (keys ? kBndK : 0);
   stamp(3);
   return true;
 }
@@ -1929,9 +1931,9 @@ __device__ __forceinline__ TileForm tile_form(const Args<T>& a, const fwh::Task&
   if (const int cap = h_clamp<BS>(ba, bb)) return {cap, 0};
   const int mode = bnd_value(ba) + bnd_value(bb) < Keys<BS>::CAP ? 1 : 0;
   int form = ((ba & kBndInf) ? kFormInfA : 0) | ((bb & kBndInf) ? kFormInfB : 0);
-  if (ba & kBndH) form |= kFormHA;
+  if (!(ba & kBndK)) form |= kFormHA;  // (16-bit keys only)
   else if (mode == 0 && bnd_value(ba) < Keys<BS>::CAP) form |= kFormKA;
-  if (bb & kBndH) form |= kFormHB;
+  if (!(bb & kBndK)) form |= kFormHB;
   else if (mode == 0 && bnd_value(bb) < Keys<BS>::CAP) form |= kFormKB;
   return {mode, form};
 }
