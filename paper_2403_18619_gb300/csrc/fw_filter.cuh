@@ -40,12 +40,11 @@ struct FilterTask {
   const T* old;          // the tile's values before, BS x BS in shared memory
   const uint32_t* Ah;    // their 16-bit bounds in shared memory
   const uint32_t* Bh;
-  const int32_t* Psrc;   // predecessors of B's rows, [kk][col]; null: via codes
+  const int32_t* Psrc;   // predecessors of B's rows, [kk][col]
   T* D;                  // the tile in the matrix
   int32_t* P;            // null: distance-only
   int64_t ld;
   int nrow, ncol, kn;    // valid rows, columns and steps
-  int r, bs;             // round, block size
   bool diag;             // the tile lies on the diagonal
   bool neg;              // an operand has a negative entry
   QScale q;
@@ -114,9 +113,9 @@ __device__ __forceinline__ void load_pair(T* dst, const T* src) {
 
 template <typename T>
 __device__ __forceinline__ void store_relaxed(const FilterTask<T>& f, int row, int col, T v,
-                                              int arg, int32_t pred) {
+                                              int32_t pred) {
   f.D[row * f.ld + col] = v;
-  if (f.P) f.P[row * f.ld + col] = f.Psrc ? pred : via_code((int64_t)f.r * f.bs + arg);
+  if (f.P) f.P[row * f.ld + col] = pred;
   if (f.diag && row == col && v < T(0)) atomicOr(f.status, kStNegCycle);
 }
 
@@ -158,7 +157,7 @@ __device__ __noinline__ void refine_many(const FilterTask<T>& f, uint32_t item, 
       }
   }
   if (arg >= 0)
-    store_relaxed(f, row, col, best, arg, f.P && f.Psrc ? __ldcg(f.Psrc + arg * BS + col) : 0);
+    store_relaxed(f, row, col, best, f.P ? __ldcg(f.Psrc + arg * BS + col) : 0);
 }
 
 // Unit halves (four steps) of a warp's many-step candidates from which on all of its
@@ -266,7 +265,7 @@ __device__ __noinline__ bool refine_list(const FilterTask<T>& f, uint32_t* list,
 #pragma unroll
     for (int u = 0; u < I; ++u)
       if (arg[u] >= 0)
-        store_relaxed(f, item[u] & 127u, item[u] >> 7 & 127u, best[u], arg[u], pred[u]);
+        store_relaxed(f, item[u] & 127u, item[u] >> 7 & 127u, best[u], pred[u]);
   }
   return true;
 }
@@ -364,11 +363,11 @@ __device__ __forceinline__ void relax_exact(const FilterTask<T>& f, int tx, int 
     int32_t pred[TM];
 #pragma unroll
     for (int nn = 0; nn < TM; ++nn)
-      pred[nn] = f.P && f.Psrc && arg[m][nn] >= 0 ? __ldcg(f.Psrc + arg[m][nn] * BS + tx * G + nn) : 0;
+      pred[nn] = f.P && arg[m][nn] >= 0 ? __ldcg(f.Psrc + arg[m][nn] * BS + tx * G + nn) : 0;
 #pragma unroll
     for (int nn = 0; nn < TM; ++nn)
       if (arg[m][nn] >= 0 && lr < f.nrow && tx * G + nn < f.ncol)
-        store_relaxed(f, lr, tx * G + nn, best[m][nn], arg[m][nn], pred[nn]);
+        store_relaxed(f, lr, tx * G + nn, best[m][nn], pred[nn]);
   }
 }
 

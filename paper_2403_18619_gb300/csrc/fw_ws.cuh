@@ -763,8 +763,6 @@ __device__ __forceinline__ FilterTask<T> filter_task(const Args<T>& a, int r, in
   f.nrow = (int)(a.n - row0 < BS ? a.n - row0 : BS);
   f.ncol = (int)(a.n - col0 < BS ? a.n - col0 : BS);
   f.kn = (int)(a.n - k0 < BS ? a.n - k0 : BS);
-  f.r = r;
-  f.bs = BS;
   f.diag = ti == tj;
   f.status = a.status;
   f.q = q_scale(__ldcg(a.qexp + r));
@@ -785,7 +783,7 @@ __device__ __forceinline__ FilterTask<T> tile_filter(const Args<T>& a, const fwh
   f.old = reinterpret_cast<const T*>(smem + L::d_off());
   f.Ah = reinterpret_cast<const uint32_t*>(smem + L::ring_off() + st * L::kStage);
   f.Bh = f.Ah + KeysH<BS>::kTileWords;
-  if (!ViaPred<T>::kOn) f.Psrc = a.rowP + tb * BS * BS;
+  f.Psrc = a.rowP + tb * BS * BS;
   f.neg = __ldcg(a.colB + ta) | __ldcg(a.rowB + tb);
   return f;
 }
@@ -883,6 +881,7 @@ template <typename T, int BS, bool kA, class Src>
 __device__ __forceinline__ int quantize_tile(uint32_t* H, const QScale& q, Src&& src) {
   using Gm = Geo<BS>;
   constexpr int G = Gm::G, NW = KeysH<BS>::kNW;
+  static_assert(NW == 2, "blocks of 64");
   int neg = 0;
 #pragma unroll 1
   for (int i = threadIdx.x; i < BS * 16; i += kThreads) {
@@ -901,9 +900,7 @@ __device__ __forceinline__ int quantize_tile(uint32_t* H, const QScale& q, Src&&
     for (int j = 0; j < 2 * NW; ++j) neg |= v[j] < T(0) ? 1 : 0;
     const int t16 = (x % Gm::SPAN) / G, m = (x / Gm::SPAN) * G + x % G;  // x = idx(t16, m)
     uint32_t* u = H + h_unit<BS>(tk * NW / 4, m, t16) + tk * NW % 4;
-    if constexpr (NW == 4) *reinterpret_cast<uint4*>(u) = make_uint4(word[0], word[1], word[2], word[3]);
-    else if constexpr (NW == 2) *reinterpret_cast<uint2*>(u) = make_uint2(word[0], word[1]);
-    else *u = word[0];
+    *reinterpret_cast<uint2*>(u) = make_uint2(word[0], word[1]);
   }
   return neg;
 }
@@ -940,7 +937,7 @@ __device__ __noinline__ bool ws_panel_f(const Args<T>& a, const fwh::Task& k, un
   FilterTask<T> f = filter_task<T, BS>(a, r, k.ti, k.tj);
   const size_t tile = (size_t)(r & 1) * a.slot_tiles + t;
   int32_t* const snapP = a.rowP + tile * BS * BS;
-  if (is_row && !ViaPred<T>::kOn && f.P) stage_tile_i32<BS>(snapP, a.P, a.n, a.ld, k.ti, k.tj, nullptr);
+  if (is_row && f.P) stage_tile_i32<BS>(snapP, a.P, a.n, a.ld, k.ti, k.tj, nullptr);
   if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns) ||
       !mbar_wait(&wb->chunk_full[s0], (pc.chunk >> 1) & 1, a.status, a.abort_flag,
                  a.timeout_ns) ||
@@ -968,7 +965,7 @@ __device__ __noinline__ bool ws_panel_f(const Args<T>& a, const fwh::Task& k, un
   f.old = own;
   f.Ah = Ah;
   f.Bh = Bh;
-  if (!ViaPred<T>::kOn) f.Psrc = is_row ? snapP : a.pivP + (size_t)(r & 1) * BS * BS;
+  f.Psrc = is_row ? snapP : a.pivP + (size_t)(r & 1) * BS * BS;
   f.neg = neg[0] != 0;
   if (!refine_tile<T, BS, false>(f, acc, tx, ty,
                                  reinterpret_cast<uint32_t*>(smem + L::scr_off() +
@@ -986,7 +983,7 @@ __device__ __noinline__ bool ws_panel_f(const Args<T>& a, const fwh::Task& k, un
   pc.chunk += 2;
   T* const snapR = (is_row ? a.rowR : a.colR) + tile * BS * BS;
   uint32_t* const snapH = (is_row ? a.rowH : a.colH) + tile * H::kTileWords;
-  if (is_row && !ViaPred<T>::kOn && f.P) stage_tile_i32<BS>(snapP, a.P, a.n, a.ld, k.ti, k.tj, nullptr);
+  if (is_row && f.P) stage_tile_i32<BS>(snapP, a.P, a.n, a.ld, k.ti, k.tj, nullptr);
   auto relaxed = [&](int i, int j) {
     const bool in = i < f.nrow && j < f.ncol;
     const T v = in ? __ldcg(f.D + i * f.ld + j) : Num<T>::inf();
