@@ -133,7 +133,7 @@ __device__ __noinline__ void refine_many(const FilterTask<T>& f, uint32_t item, 
   int arg = -1;
   // a unit half (four steps) at a time, its operands loaded together
   while (flags) {
-    int kk[4];
+    int kk[4] = {0, 0, 0, 0};  // n of them
     int n = 0;
     next_hits<BS>(flags, pa, pb, thr, [&](int k) {
       kk[0] = n == 0 ? k : kk[0];
