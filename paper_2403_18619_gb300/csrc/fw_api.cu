@@ -113,13 +113,13 @@ int kernel_setup(const void* fn, size_t smem, int threads) {
   return occ;
 }
 
-size_t solve_ws_bytes(int R, int BS, int esize) {
+size_t solve_ws_bytes(int R, int BS, int esize, bool filtered) {
   const size_t t = (size_t)BS * BS;
-  const size_t keys = esize == 4 ? 2 : 1;  // packed-key (64-bit elements: 16-bit) snapshots
+  const size_t keys = esize == 4 ? 2 : filtered ? 1 : 0;  // packed-key snapshots, or 16-bit bounds
   size_t b = 0;
   b += up(((size_t)R * R + 2 * (size_t)R) * 4 + 4 * 4 + 4);  // ver + done + ctr + abort
   b += up((size_t)(R + 2) * 4);              // stage offsets
-  b += up((size_t)R * 4);                    // exponents of the 16-bit bounds
+  if (filtered) b += up((size_t)R * 4);      // exponents of the 16-bit bounds
   b += up(2 * t * esize) + up(2 * t * 4);    // piv, pivP
   b += up(2 * (size_t)R * t * 4) * keys;     // colK, rowK
   b += up(2 * (size_t)R * t * esize) * 2;    // colR, rowR
@@ -128,7 +128,7 @@ size_t solve_ws_bytes(int R, int BS, int esize) {
   return b + kAlign;
 }
 
-SolveWs carve_solve_ws(void* base, int R, int BS, int esize) {
+SolveWs carve_solve_ws(void* base, int R, int BS, int esize, bool filtered) {
   SolveWs w;
   char* p = reinterpret_cast<char*>((reinterpret_cast<uintptr_t>(base) + kAlign - 1) / kAlign * kAlign);
   const size_t t = (size_t)BS * BS;
@@ -139,10 +139,14 @@ SolveWs carve_solve_ws(void* base, int R, int BS, int esize) {
   w.flags_bytes = ((size_t)R * R + 2 * (size_t)R) * 4 + 4 * 4 + 4;
   p += up(w.flags_bytes);
   w.stage_off = reinterpret_cast<unsigned*>(p);  p += up((size_t)(R + 2) * 4);
-  w.qexp = reinterpret_cast<int*>(p);            p += up((size_t)R * 4);
+  if (filtered) {
+    w.qexp = reinterpret_cast<int*>(p);          p += up((size_t)R * 4);
+  }
   w.piv = p;                                     p += up(2 * t * esize);
   w.pivP = reinterpret_cast<int32_t*>(p);        p += up(2 * t * 4);
-  w.colK = reinterpret_cast<uint32_t*>(p);       p += up(2 * (size_t)R * t * 4);
+  if (esize == 4 || filtered) {
+    w.colK = reinterpret_cast<uint32_t*>(p);     p += up(2 * (size_t)R * t * 4);
+  }
   if (esize == 4) {
     w.rowK = reinterpret_cast<uint32_t*>(p);     p += up(2 * (size_t)R * t * 4);
   }
@@ -245,9 +249,10 @@ fw_status solve_device(void* dist, int32_t* pred, int64_t n, int64_t ld, fw_dtyp
   StreamWs* w = nullptr;
   auto lk = lock_entry(s, &w);
   if (!w) return FW_ERR_CUDA;
-  fw_status st = get_ws(*w, s, solve_ws_bytes(R, BS, esize));
+  const bool filtered = filtered_tiles(dtype == FW_F64, BS);
+  fw_status st = get_ws(*w, s, solve_ws_bytes(R, BS, esize, filtered));
   if (st != FW_OK) return st;
-  SolveWs ws = carve_solve_ws(w->base, R, BS, esize);
+  SolveWs ws = carve_solve_ws(w->base, R, BS, esize, filtered);
   ws.status = w->status;
   if (w->cached_R != R || w->cached_BS != BS || w->cached_look != look) {
     std::vector<unsigned> off(R + 2);
@@ -509,7 +514,9 @@ fw_status fw_solve_plan(int64_t n, fw_dtype dtype, const fw_options* opt, int32_
   if (bs) *bs = BS;
   if (rounds) *rounds = R;
   if (lookahead) *lookahead = o.lookahead < 0 ? auto_lookahead(R, sms) : o.lookahead;
-  if (workspace_bytes) *workspace_bytes = (int64_t)solve_ws_bytes(R, BS, dtype_size(dtype));
+  if (workspace_bytes)
+    *workspace_bytes = (int64_t)solve_ws_bytes(R, BS, dtype_size(dtype),
+                                               filtered_tiles(dtype == FW_F64, BS));
   return FW_OK;
 }
 

@@ -37,6 +37,8 @@
 #include <type_traits>
 #include <utility>
 
+#include "fw_internal.h"
+
 namespace fwk {
 
 constexpr int kThreads = 256;
@@ -356,7 +358,7 @@ __device__ __forceinline__ T vmin(T a, T b) {
 // ms).  int64 relaxes a tile in 36 K cycles; filtered, n = 1000 went from 1.34 to
 // 2.13 ms and n = 3000 only from 12.9 to 11.8.
 template <typename T, int BS>
-constexpr bool kFiltered = std::is_same<T, double>::value && BS == 64;
+constexpr bool kFiltered = fwh::filtered_tiles(std::is_same<T, double>::value, BS);
 
 // q = floor(v * 2^e) of the filtered min-plus (fw_filter.cuh): 0 .. kQMax, a
 // larger finite value kQMax, a negative one 0, INF kQInf.
@@ -540,7 +542,7 @@ struct Args {
 // Snapshot pointers of a workspace.  The 16-bit snapshots (2 bytes per entry,
 // two panels) of an int32 solve fill the array of row-panel predecessors, which
 // it does not keep (via codes); fp64 has an array of that size for its 16-bit
-// bounds. 
+// bounds where it uses them.
 template <typename T, class Ws>
 void set_snapshots(Args<T>& a, const Ws& ws) {
   a.slot_tiles = ws.slot_tiles;
@@ -548,7 +550,8 @@ void set_snapshots(Args<T>& a, const Ws& ws) {
   a.colK = ws.colK; a.colR = reinterpret_cast<T*>(ws.colR); a.colB = ws.colB;
   a.rowK = ws.rowK; a.rowR = reinterpret_cast<T*>(ws.rowR); a.rowP = ws.rowP; a.rowB = ws.rowB;
   a.colH = Num<T>::kPacked ? reinterpret_cast<uint32_t*>(ws.rowP) : ws.colK;
-  a.rowH = a.colH + (size_t)ws.R * ws.BS * ws.BS;  // 2 slots x R tiles x BS^2 / 2 words
+  // (2 slots x R tiles x BS^2 / 2 words)
+  a.rowH = a.colH ? a.colH + (size_t)ws.R * ws.BS * ws.BS : nullptr;
   a.qexp = ws.qexp;
 }
 

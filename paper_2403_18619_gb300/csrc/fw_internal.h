@@ -131,7 +131,7 @@ struct SolveWs {
   int* abort_flag = nullptr;
   int* status = nullptr;
   unsigned* stage_off = nullptr;
-  int* qexp = nullptr;  // [R] exponents of the 16-bit bounds
+  int* qexp = nullptr;  // [R] exponents of the 16-bit bounds (filtered tiles)
   void* piv = nullptr;
   int32_t* pivP = nullptr;
   uint32_t* colK = nullptr;
@@ -145,12 +145,15 @@ struct SolveWs {
   size_t flags_bytes = 0;  // ver + done + ctr + abort (zeroed before each solve)
 };
 
+// Whether tiles are filtered by 16-bit bounds (fw_device.cuh, kFiltered).
+__host__ __device__ constexpr bool filtered_tiles(bool fp64, int BS) { return fp64 && BS == 64; }
+
 // Bytes needed by a solve of R tiles of BS with esize-byte elements (4: int32
-// or fp32, with the packed-key snapshots; 8: int64 or fp64, with one array of
-// that size for their 16-bit snapshots).
-size_t solve_ws_bytes(int R, int BS, int esize = 4);
+// or fp32, with the packed-key snapshots; 8: int64 or fp64, with the 16-bit
+// bounds in an array of that size where tiles are filtered).
+size_t solve_ws_bytes(int R, int BS, int esize = 4, bool filtered = false);
 // Carve a workspace out of `base` (cudaMalloc'd, >= solve_ws_bytes).
-SolveWs carve_solve_ws(void* base, int R, int BS, int esize = 4);
+SolveWs carve_solve_ws(void* base, int R, int BS, int esize = 4, bool filtered = false);
 
 struct LaunchCfg {
   int BS;
