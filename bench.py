@@ -10,8 +10,9 @@ relaxations.  The metric is relaxations per second, n^3 / t.
 Prints one JSON line.  `value` times the solve with the input already in HBM
 (the input is restored from a pristine device copy before every step, outside
 the timed events); `e2e` times fw_solve_host_io (the weights from one pinned
-host buffer, the results into others), copies included.  `roofline` compares the persistent solver kernel against the
-min-plus relaxation peak measured by fw_peak_probe in the same process.  The
+host buffer, the results into others), copies included.  `roofline` compares the
+persistent solver kernel against the min-plus relaxation peak over 16-bit keys
+(path_peak), the fastest loop its tiles take, measured in the same process.  The
 CPU baseline is the oracle's plain triple loop on a bounded sample of the same
 workload.  With --impl reference the oracle alone is timed the same way.
 Under torchrun every rank solves its own instance (independent replicas; the
@@ -40,11 +41,11 @@ BS = 128
 SAMPLE_N = 2048          # CPU baseline: leading 2048-vertex induced subgraph
 # DRAM bytes (read + write) of one k_persistent_ws launch of the current
 # kernel, keyed by (n, BS, driver); null in the line where no capture exists.
-# n = 32768: one ncu capture of the same kernel at n = 16384 (339.4e9 B)
+# n = 32768: one ncu capture of the same kernel at n = 16384 (332.7e9 B)
 # scaled by n^3; an upper bound, since the bytes above the algorithmic
 # 8 n^3 / BS (2.20e12 B here) are scattered predecessor stores whose share
-# falls as n grows (1.29x at n = 8192, 1.23x at n = 16384).
-TRAFFIC_BYTES = {(32768, 128, 1): 339.4e9 * 8}
+# falls as n grows (1.26x at n = 8192, 1.21x at n = 16384).
+TRAFFIC_BYTES = {(32768, 128, 1): 332.7e9 * 8}
 TRAFFIC_NOTE = {(32768, 128, 1): "ncu dram bytes of one launch at n = 16384, scaled by n^3 "
                                  "(upper bound; algorithmic 8 n^3 / BS = 2.20e12 B)"}
 
@@ -300,7 +301,7 @@ def bench_batched(fw, args):
     t_single = a.elapsed_time(b)
     plan.close()
     relax = float(sum(int(n) ** 3 for n in ns))
-    peak = fw.fw_peak_probe(fw.FW_I32)[0]
+    peak = path_peak(fw, fw.FW_I32)[0]
     return {"workload": "512 digraphs, n ~ U[64,2048] (seed 11), p=0.3, int32 U[1,100]",
             "graphs_per_s": 512 / (t_batched * 1e-3), "relax_per_s": relax / (t_batched * 1e-3),
             "frac_of_peak": relax / (t_batched * 1e-3) / peak, "peak_relax_per_s": peak,
@@ -308,6 +309,15 @@ def bench_batched(fw, args):
             "speedup_vs_one_launch_per_graph": t_single / t_batched,
             "bs_table": table.tolist(), "tasks": int(ntasks),
             "timing": "events around fw_solve_batched (graph replay); inputs restored outside"}
+
+
+def path_peak(fw, dtype):
+    """(relaxations/s, relaxations per SM clock, SM MHz, name) of the loop that bounds
+    a solve of this type: over 16-bit keys for int32 and for fp64 (whose blocks of
+    64 filter their relaxations through it), else the type's own add and min."""
+    if dtype in (fw.FW_I32, fw.FW_F64):
+        return fw.fw_peak_probe_keys16() + ("fw_peak_probe_keys16, __viaddmin_u16x2",)
+    return fw.fw_peak_probe(dtype) + ("fw_peak_probe, add + min",)
 
 
 def _peaks():
@@ -514,8 +524,8 @@ def bench_configs(fw, args, only=None):
     """The other single-graph workloads: n = 1024 complete digraph, int32
     U[1,100], BS = 32 (launch / latency-bound), and n = 8192, p = 0.5, as fp32
     (0,1] (with and without predecessors), int32 U[1,1000], fp64 (0,1] and
-    int64 U[1,1e12], each against its own measured peak (fw_peak_probe of its
-    dtype)."""
+    int64 U[1,1e12], each against the measured peak of the loop that bounds it
+    (path_peak)."""
     import torch
     import graphgen.device as gdev
     out = {}
@@ -524,14 +534,14 @@ def bench_configs(fw, args, only=None):
         if only is not None and name != only:
             continue
         if dt not in peaks:
-            peaks[dt] = fw.fw_peak_probe(dt)[0]
+            peaks[dt] = path_peak(fw, dt)
         ld = fw.padded(n)
         W = torch.empty((n, ld), dtype=_torch_dtype(fw, dt), device="cuda")
         _fill(fw, dt)(W[:, :n], seed=seed, p=p, **gen)
         D = torch.empty_like(W)
         P = torch.empty((n, ld), dtype=torch.int32, device="cuda")
         opt = fw.Options.default(bs=bs)
-        # the fp64 solve runs on GB300's narrow FP64 pipe (about 1 s at n = 8192)
+        # the fp64 solve is the slowest (about 0.15 s at n = 8192)
         steps = 3 if dt == fw.FW_F64 else max(3, args.steps)
         ts = []
         for i in range(2 + steps):
@@ -545,8 +555,9 @@ def bench_configs(fw, args, only=None):
                 ts.append(a.elapsed_time(b))
         t = sorted(ts)[len(ts) // 2]
         rps = n ** 3 / (t * 1e-3)
-        out[name] = {"ms_median": t, "relax_per_s": rps, "frac_of_peak": rps / peaks[dt],
-                     "peak_relax_per_s": peaks[dt], "steps": steps}
+        out[name] = {"ms_median": t, "relax_per_s": rps, "frac_of_peak": rps / peaks[dt][0],
+                     "peak_relax_per_s": peaks[dt][0], "peak_source": peaks[dt][3],
+                     "steps": steps}
         del W, D, P
     return out
 
@@ -574,7 +585,8 @@ def run_gpu(args):
     D = torch.empty_like(W)
     P = torch.empty((n, ld), dtype=torch.int32, device="cuda")
 
-    rps, per_clk, probe_mhz = fw.fw_peak_probe(fw.FW_I32)
+    rps, per_clk, probe_mhz, probe = path_peak(fw, fw.FW_I32)
+    rps32 = fw.fw_peak_probe(fw.FW_I32)[0]
 
     ev0 = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
     ev1 = [torch.cuda.Event(enable_timing=True) for _ in range(args.steps)]
@@ -669,9 +681,10 @@ def run_gpu(args):
                      "traffic": TRAFFIC_BYTES.get((n, args.bs, args.driver)),
                      "traffic_source": TRAFFIC_NOTE.get((n, args.bs, args.driver)),
                      "kernel": "k_persistent_ws<int,128>",
-                     "peak_source": "fw_peak_probe (__viaddmin_u32 chains on all SMs, same "
-                                    "process, %.1f relax/SM-clk at %.0f MHz)" % (per_clk,
-                                                                                  probe_mhz)},
+                     "peak_keys32": rps32 / 1e12,
+                     "peak_source": "%s chains on all SMs, same process, %.1f relax/SM-clk at "
+                                    "%.0f MHz; peak_keys32: __viaddmin_u32" % (probe, per_clk,
+                                                                               probe_mhz)},
         "clocks": clocks.summary(),
         "gpu_launches": 3 * args.steps,  # init, persistent solver, predecessor resolution
         "wall_s_timed_region": wall,

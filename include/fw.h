@@ -288,14 +288,22 @@ fw_status fw_release_workspace(void);
 
 /*
  * fw_peak_probe: measures the min-plus relaxation peak of this GPU at its
- * current clocks with register-resident relaxation chains on every SM (the
- * same instruction the solver's inner loop issues: __viaddmin for int32,
- * add + min for fp32, fp64 and int64).  Outputs relaxations per second, relaxations per SM
- * clock cycle (clock-independent) and the average SM clock in MHz seen by the
- * probe.  Synchronous.  Not part of the paper: it provides the roofline.
+ * current clocks with register-resident relaxation chains on every SM: one
+ * 32-bit __viaddmin per relaxation for int32 (the solver's loop over 32-bit
+ * keys), add + min for fp32, fp64 and int64.  Outputs relaxations per second,
+ * relaxations per SM clock cycle (clock-independent) and the average SM clock
+ * in MHz seen by the probe.  Synchronous.  Not part of the paper: it provides
+ * the roofline.
+ *
+ * fw_peak_probe_keys16: the same for the loop over 16-bit keys, two relaxations
+ * per __viaddmin_u16x2.  It bounds int32 solves, whose tiles take that loop where
+ * their distances allow it, and fp64 solves in blocks of 64, which filter their
+ * relaxations through it.
  */
 fw_status fw_peak_probe(fw_dtype dtype, double* relax_per_s, double* relax_per_sm_clk,
                         double* sm_mhz, void* stream);
+fw_status fw_peak_probe_keys16(double* relax_per_s, double* relax_per_sm_clk, double* sm_mhz,
+                               void* stream);
 
 /*
  * fw_verify_certificate: GPU check of the LP-duality certificate of exact

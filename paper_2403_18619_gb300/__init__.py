@@ -17,7 +17,8 @@ import numpy as np
 __all__ = [
     "FWError", "Options", "load", "check", "fw_solve", "fw_solve_ex", "fw_solve_host",
     "fw_solve_host_io", "fw_solve_noalloc", "fw_sync_status", "fw_backward", "fw_backward_strided",
-    "fw_peak_probe", "fw_verify_certificate", "fw_release_workspace", "fw_solve_plan",
+    "fw_peak_probe", "fw_peak_probe_keys16", "fw_verify_certificate", "fw_release_workspace",
+    "fw_solve_plan",
     "fw_queue_tasks", "fw_batched_task_list", "fw_paths", "fw_intermediate", "fw_tile_closure", "fw_tile_minplus", "fw_block_init_pred",
     "BatchedPlan", "fw_bs_table", "fw_autotune_bs", "padded", "solve",
     "solve_batched", "INF_I32", "INF_I64", "FW_I32", "FW_F32", "FW_I64", "FW_F64", "DRIVER_AUTO",
@@ -104,6 +105,7 @@ def load():
         lib.fw_sync_status.argtypes = [P]
         lib.fw_release_workspace.argtypes = []
         lib.fw_peak_probe.argtypes = [I32, P, P, P, P]
+        lib.fw_peak_probe_keys16.argtypes = [P, P, P, P]
         lib.fw_verify_certificate.argtypes = [P, P, P, I64, I64, P, P]
         lib.fw_queue_tasks.argtypes = [I32, I64, I64, I64, P]
         lib.fw_batched_task_list.argtypes = [P, P, I64, I32, P, P, I64, P]
@@ -122,8 +124,8 @@ def load():
                      "fw_batched_plan_create",
                      "fw_solve_batched", "fw_batched_plan_info", "fw_batched_plan_destroy",
                      "fw_backward", "fw_backward_strided", "fw_sync_status",
-                     "fw_release_workspace", "fw_peak_probe", "fw_verify_certificate",
-                     "fw_queue_tasks", "fw_batched_task_list", "fw_solve_noalloc", "fw_bs_table",
+                     "fw_release_workspace", "fw_peak_probe", "fw_peak_probe_keys16",
+                     "fw_verify_certificate", "fw_queue_tasks", "fw_batched_task_list", "fw_solve_noalloc", "fw_bs_table",
                      "fw_autotune_bs",
                      "fw_solve_plan", "fw_paths", "fw_intermediate", "fw_tile_closure",
                      "fw_tile_minplus",
@@ -291,6 +293,14 @@ def fw_peak_probe(dtype: int = FW_I32, stream=None):
     a, b, c = ctypes.c_double(), ctypes.c_double(), ctypes.c_double()
     check(load().fw_peak_probe(dtype, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c),
                                _stream_ptr(stream)), "fw_peak_probe")
+    return a.value, b.value, c.value
+
+
+def fw_peak_probe_keys16(stream=None):
+    """fw_peak_probe over 16-bit keys: two relaxations per instruction."""
+    a, b, c = ctypes.c_double(), ctypes.c_double(), ctypes.c_double()
+    check(load().fw_peak_probe_keys16(ctypes.byref(a), ctypes.byref(b), ctypes.byref(c),
+                                      _stream_ptr(stream)), "fw_peak_probe_keys16")
     return a.value, b.value, c.value
 
 

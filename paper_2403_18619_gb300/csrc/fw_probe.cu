@@ -2,9 +2,12 @@
 //
 // Each thread keeps a block of relaxation chains in registers (8 x 8 for the
 // 32-bit types, 1 x 8 for the 64-bit ones, so that 512 threads fit the
-// register file) and relaxes it with the instructions the solver issues per
-// relaxation:
-//   int32 : acc = __viaddmin_u32(a, b, acc)     (one DPX instruction)
+// register file) and relaxes it:
+//   int32 : acc = __viaddmin_u32(a, b, acc)     (one DPX instruction, as the solver
+//                                                over 32-bit keys)
+//   16-bit: acc = __viaddmin_u16x2(a, b, acc)   (one DPX instruction for two, as the
+//                                                solver over 16-bit keys and the
+//                                                16-bit bounds of fp64)
 //   fp32  : acc = fminf(a + b, acc)             (add + min)
 //   fp64  : acc = a + b < acc ? a + b : acc     (DADD, then an integer min of
 //                                                the bit patterns, as the solver)
@@ -30,9 +33,11 @@ template <> struct ProbeMode<float> { static constexpr int M = 8; };
 template <> struct ProbeMode<double> { static constexpr int M = 1; };
 template <> struct ProbeMode<int64_t> { static constexpr int M = 1; };
 
-template <typename T>
+template <typename T, bool kPairs>
 __device__ __forceinline__ T relax(T a, T b, T acc) {
-  if constexpr (std::is_same<T, uint32_t>::value) {
+  if constexpr (kPairs) {
+    return __viaddmin_u16x2(a, b, acc);
+  } else if constexpr (std::is_same<T, uint32_t>::value) {
     return __viaddmin_u32(a, b, acc);
   } else if constexpr (std::is_same<T, float>::value) {
     return fminf(a + b, acc);
@@ -53,7 +58,7 @@ __device__ __forceinline__ T seed_value(uint32_t s, int k) {
   else return (int64_t)s * 1000003ll + k;
 }
 
-template <typename T>
+template <typename T, bool kPairs = false>
 __global__ void __launch_bounds__(kProbeThreads, 1)
     k_probe(const uint32_t* __restrict__ seed, uint32_t* __restrict__ sink, int iters,
             long long* __restrict__ cycles) {
@@ -79,7 +84,7 @@ __global__ void __launch_bounds__(kProbeThreads, 1)
 #pragma unroll
       for (int m = 0; m < M; ++m)
 #pragma unroll
-        for (int n = 0; n < 8; ++n) acc[m][n] = relax<T>(a[m], b[u][n], acc[m][n]);
+        for (int n = 0; n < 8; ++n) acc[m][n] = relax<T, kPairs>(a[m], b[u][n], acc[m][n]);
 #pragma unroll
     for (int m = 0; m < M; ++m) a[m] = acc[m][m];
   }
@@ -100,11 +105,9 @@ __global__ void __launch_bounds__(kProbeThreads, 1)
   if (threadIdx.x == 0) cycles[blockIdx.x] = c1 - c0;
 }
 
-}  // namespace
-
-extern "C" fw_status fw_peak_probe(fw_dtype dtype, double* relax_per_s, double* relax_per_sm_clk,
-                                   double* sm_mhz, void* stream) {
-  if (dtype != FW_I32 && dtype != FW_F32 && dtype != FW_I64 && dtype != FW_F64) return FW_ERR_ARG;
+// pairs: over 16-bit keys (dtype FW_I32).
+fw_status probe(fw_dtype dtype, bool pairs, double* relax_per_s, double* relax_per_sm_clk,
+                double* sm_mhz, void* stream) {
   cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
   const int sms = fwh::num_sms();
   uint32_t *seed = nullptr, *sink = nullptr;
@@ -126,8 +129,9 @@ extern "C" fw_status fw_peak_probe(fw_dtype dtype, double* relax_per_s, double* 
     // the 64-bit pipes are far slower: fewer iterations for a similar duration
     const bool wide = dtype == FW_I64 || dtype == FW_F64;
     const int iters = wide ? 1 << 13 : 1 << 15;
-    const int chains = wide ? 8 : 64;
-    auto kern = dtype == FW_I32   ? k_probe<uint32_t>
+    const int chains = wide ? 8 : pairs ? 128 : 64;
+    auto kern = pairs             ? k_probe<uint32_t, true>
+                : dtype == FW_I32 ? k_probe<uint32_t>
                 : dtype == FW_F32 ? k_probe<float>
                 : dtype == FW_F64 ? k_probe<double>
                                   : k_probe<int64_t>;
@@ -158,4 +162,17 @@ extern "C" fw_status fw_peak_probe(fw_dtype dtype, double* relax_per_s, double* 
   if (sink) cudaFree(sink);
   if (cyc) cudaFree(cyc);
   return st;
+}
+
+}  // namespace
+
+extern "C" fw_status fw_peak_probe(fw_dtype dtype, double* relax_per_s, double* relax_per_sm_clk,
+                                   double* sm_mhz, void* stream) {
+  if (dtype != FW_I32 && dtype != FW_F32 && dtype != FW_I64 && dtype != FW_F64) return FW_ERR_ARG;
+  return probe(dtype, false, relax_per_s, relax_per_sm_clk, sm_mhz, stream);
+}
+
+extern "C" fw_status fw_peak_probe_keys16(double* relax_per_s, double* relax_per_sm_clk,
+                                          double* sm_mhz, void* stream) {
+  return probe(FW_I32, true, relax_per_s, relax_per_sm_clk, sm_mhz, stream);
 }
