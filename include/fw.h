@@ -92,7 +92,7 @@ typedef struct fw_options {
   int32_t driver;             /* fw_driver */
   int32_t lookahead;          /* persistent driver: remaining-block tasks of round r queued
                                  between the pivot and the panels of round r+1; -1 = automatic
-                                 (six per CTA, fewer when a round has few tasks) */
+                                 (six per SM, fewer when a round has few tasks) */
   int32_t grid;               /* persistent driver: CTAs; 0 = every co-resident CTA */
   int64_t timeout_ns;         /* bound on one device-side dependency wait; 0 = 2 s */
   int32_t packed_keys;        /* int32 only: 1 (default) relaxes packed (distance, pivot) keys
@@ -107,8 +107,8 @@ typedef struct fw_options {
                                  (claim, inputs ready, operands issued, published; compute start
                                  and end), the GPU view of the idle time Opt-9 targets (Sec. 4.3).
                                  Min-plus tasks add SM-cycle counts: column 7 = tile-load wait |
-                                 operand-chunk waits << 20 | predecessor-tile wait << 40 (20 bits
-                                 each, saturating), column 8 = cycles from task start to the end
+                                 operand-chunk waits << 20 (20 bits each, saturating; the 20 bits
+                                 above, a wait for a predecessor tile, stay 0), column 8 = cycles from task start to the end
                                  of the relaxation | whole task << 32.  Pivot and panel tasks:
                                  column 7 = operands loaded | relaxed << 32, column 8 = results
                                  stored | whole task << 32 (SM cycles from the task's start).

@@ -159,11 +159,13 @@ SolveWs carve_solve_ws(void* base, int R, int BS, int esize, bool filtered) {
   return w;
 }
 
-// Automatic BS of a single solve.  Larger blocks relax faster (BS = 128 runs
-// the DPX loop at ~84 % of peak, BS = 64 at ~50 %) but make R = n / BS rounds
-// whose pivot -> panel chain is longer; measured on GB300 (int32, persistent
-// driver): n = 2048 BS 64 1.27 ms vs BS 128 2.16 ms; n = 4096 BS 64 7.70 ms vs
-// BS 128 5.91 ms.  The two costs cross near n = 3072.
+// Automatic BS of a single solve.  Larger blocks relax faster but make R = n / BS
+// rounds whose pivot -> panel chain is longer.  Measured on GB300 (ms, persistent
+// driver, p = 0.5, with predecessors; BS 32 / 64): n = 512 int32 0.35 / 0.35, fp32
+// 0.32 / 0.36; n = 1024 0.64 / 0.59 and 0.64 / 0.66.  BS 64 / 128: int32 n = 2048
+// 1.13 / 1.73, 3072 2.35 / 2.63, 3584 3.46 / 3.37, 4096 5.03 / 4.56; fp32 3072
+// 4.31 / 5.60, 3584 6.70 / 7.63, 4096 9.91 / 10.4.  The line at 3072 dates from int32
+// over 32-bit keys; the costs now cross near n = 3500 (int32) and 4300 (fp32).
 int pick_bs(int64_t n, fw_dtype dtype = FW_I32) {
   if (n <= 512) return 32;
   if (n <= 3072 || dtype == FW_I64 || dtype == FW_F64) return 64;

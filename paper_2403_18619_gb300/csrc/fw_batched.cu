@@ -116,8 +116,8 @@ constexpr int kClasses = 7;  // n <= 128, 256, 512, 1024, 2048, 4096, larger
 const int64_t kClassMax[kClasses] = {128, 256, 512, 1024, 2048, 4096, 1 << 30};
 
 // One table per element type (int32, fp32): the defaults are fw_autotune_bs's
-// choices on GB300 (16 graphs per class); packed int32 keys favour BS = 128
-// down to the smallest class, fp32's three-instruction relaxation BS = 32.
+// choices on GB300 (16 graphs per class) over 32-bit keys; over 16-bit ones it takes
+// 128 for int32 graphs of 257 to 512 vertices as well, and the same for the rest.
 std::mutex g_table_mu;
 int g_bs_table[2][kClasses] = {{128, 64, 64, 128, 128, 128, 128},
                                {32, 64, 64, 128, 128, 128, 128}};

@@ -24,7 +24,11 @@
 //     finite entry of the two operand tiles is bounded so that their sums stay
 //     below CAP; each panel tile carries that bound, and a task whose operands
 //     exceed it falls back to the generic kernel (distance compare + argmin
-//     select per relaxation), which is also the fp32 kernel.
+//     select per relaxation).  The persistent driver relaxes over 16-bit keys, two
+//     steps per instruction, where the bounds allow those (KeysH).
+//   * fp32 is relaxed in groups of four steps (fw_quad.cuh), fp64 in blocks of 64
+//     through a filter of 16-bit bounds (fw_filter.cuh), int64 and small fp64 by the
+//     generic kernel; the phased driver's floating tiles and 64-bit ones by the latter.
 //   * Panel outputs are copied into double-buffered "snapshots" (already in
 //     A-form / B-form and in packed-key encoding) that phase-4 tasks stream
 //     into shared memory with cp.async.bulk (TMA), so that the next round may
@@ -352,7 +356,7 @@ __device__ __forceinline__ T vmin(T a, T b) {
 // Whether the remaining tiles and panels are filtered by 16-bit bounds
 // (fw_filter.cuh): fp64 in blocks of 64.  Its exact relaxation of a tile takes
 // 160 K SM cycles there, the filtered one 20-60 K after the first rounds (n = 700:
-// 2.87 -> 2.01 ms, n = 4096: 133 -> 26.3 ms); tiles whose bounds say little are
+// 2.87 -> 1.98 ms, n = 4096: 133 -> 25.4 ms); tiles whose bounds say little are
 // relaxed exactly after all.  At BS = 32 (n <= 512) a tile takes 19 K cycles and the rounds are
 // bound by their chain, which filtered panels lengthen (n = 400: 0.59 -> 0.68
 // ms).  int64 relaxes a tile in 36 K cycles; filtered, n = 1000 went from 1.34 to
@@ -945,8 +949,8 @@ __device__ __forceinline__ void argmin_finish(int (&arg)[TM][TM]) {
 }
 
 // Generic relaxation with an explicit first-argmin: s = A + B; if (s < acc)
-// { acc = s; arg = kk + 1 }.  Used for fp32, the 64-bit types and int32
-// tiles whose values exceed the packed-key bound.
+// { acc = s; arg = kk + 1 }.  Used for int64, fp64 in blocks of 32 and int32 tiles
+// whose values exceed the packed-key bound, and by the phased driver for all types.
 //
 // fp32 keeps the argmin on the FMA pipe: while the steps run, arg holds the
 // bits of a float accumulator to which every improving step k = kk0 + kk adds

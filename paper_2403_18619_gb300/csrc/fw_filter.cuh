@@ -315,8 +315,8 @@ __device__ __forceinline__ int find_candidates(const FilterTask<T>& f,
 // far less than the narrow FP64 pipe leaves time for).  Bound by that pipe, as the
 // exact kernel: with a vertex at 1e9 in every block of 64 and its edges as likely
 // as not, n = 4096 took 405 ms when every entry was refined step by step, 133 with
-// the exact kernel, 71 now (n = 2048: 52, 17.1, 10.7; n = 1500: 23.1, 7.6, 7.0;
-// n = 700: 9.8, 2.87, 2.87).
+// the exact kernel, 70.5 now (n = 2048: 52, 17.1, 10.5; n = 1500: 23.1, 7.6, 7.4;
+// n = 700: 9.8, 2.87, 2.85).
 template <typename T, int BS, bool kGmem>
 __device__ __forceinline__ void relax_exact(const FilterTask<T>& f, int tx, int ty) {
   using Gm = Geo<BS>;

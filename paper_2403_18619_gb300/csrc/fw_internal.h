@@ -30,12 +30,16 @@ __host__ __device__ inline int64_t size_L(int R, int r) { return (r + 1 < R) ? 2
 __host__ __device__ inline int64_t size_rest(int R, int r) {
   return (int64_t)(R - 1) * (R - 1) - size_L(R, r);
 }
-// Automatic lookahead g for `sms` co-resident CTAs: enough remaining tiles
+// Automatic lookahead g on a GPU of `sms` SMs: enough remaining tiles
 // of round s-1 ahead of the panels of round s that the panels are claimed as
 // the pivot finishes (its inputs' wait plus the pivot itself last about six
-// BS = 128 remaining-tile tasks; claimed earlier, a panel task idles its SM
-// until then), while leaving at least three tasks per CTA behind the panels
-// to cover their own latency before round s's remaining tiles need them.
+// BS = 128 remaining-tile tasks over 32-bit keys, eight to ten over 16-bit ones;
+// claimed earlier, a panel task idles its SM until then), while leaving at least
+// three tasks per SM behind the panels to cover their own latency before round s's
+// remaining tiles need them.  ms at 2 / 4 / 6 / 8 / 12 tasks per SM ahead (int32,
+// weights to 1000): n = 4096 4.46 / 4.41 / 4.62 / 4.62 / 4.64 (the rule takes 444
+// tasks: 4.50), n = 8192 24.6 / 23.4 / 22.4 / 21.8 / 21.7, n = 16384 173 / 170.5 /
+// 167.7 / 167.4 / 167.4.
 __host__ __device__ inline int64_t auto_lookahead(int R, int sms) {
   const int64_t nrest = size_rest(R, 0);
   int64_t g = nrest - 3 * (int64_t)sms;

@@ -835,7 +835,7 @@ __device__ __noinline__ bool ws_exact_f(const Args<T>& a, const fwh::Task& k, un
 // Remaining-tile task of fp64 (BS = 64): the 16-bit pass in turns, then the exact
 // relaxation of the entries that may improve while the other group of warps has
 // its turn.  The first rounds are bound by those relaxations, the later ones by the
-// 16-bit pass (20 K SM cycles per tile, exact 160 K): n = 4096 133 -> 27 ms.
+// 16-bit pass (20 K SM cycles per tile, exact 160 K): n = 4096 133 -> 25.4 ms.
 template <typename T, int BS, int LBS>
 __device__ __noinline__ bool ws_minplus_f(const Args<T>& a, const fwh::Task& k, unsigned char* smem,
                                           WsBars* wb, PipeCnt& pc, uint64_t* tr, bool& exact) {
@@ -1023,8 +1023,8 @@ __device__ __forceinline__ bool ws_minplus_body(TileCtx<T> c, int ti, int tj, in
   const int ncol = (int)(c.n - col0 < BS ? c.n - col0 : BS);
   const bool full = nrow == BS && ncol == BS;
 
-  // optional per-phase SM-cycle counts (trace): Dbuf wait, operand-chunk
-  // waits, predecessor-tile wait; start to end of the relaxation, whole task
+  // optional per-phase SM-cycle counts (trace): Dbuf wait, operand-chunk waits;
+  // start to end of the relaxation, whole task
   const long long t_a = tr ? clock64() : 0;
   long long cw = 0;
   // 1. the tile's current values (rows/columns beyond n read as INF)
@@ -2387,8 +2387,9 @@ __global__ void __launch_bounds__(kWsThreads, kCtas)
 // pivots waits for.  From 12 tiles per SM and round on the first counts more (one /
 // two CTAs per SM, int32 R = 36 1.34 / 1.42 ms, R = 41 1.83 / 1.77, R = 47 2.62 /
 // 2.22; weights to 3e5, R = 41 1.91 / 1.92, R = 47 2.75 / 2.60; fp32 R = 36 2.15 /
-// 2.17, R = 41 3.04 / 2.79, R = 47 4.53 / 4.26).  The kernel for one CTA keeps its
-// 168 registers (at 102 it is 2 % slower: n = 1000 0.60 -> 0.61 ms).
+// 2.17, R = 41 3.04 / 2.79, R = 47 4.53 / 4.26).  Two CTAs leave a thread 96
+// registers; the kernel for one uses 129 (int32) or 134 (fp32), and at 96 it is 2 %
+// slower (n = 1000 0.60 -> 0.61 ms).
 template <typename T, int BS>
 auto persistent_kernel(int R) {
   if constexpr (BS == 64 && sizeof(T) == 4)

@@ -15,7 +15,8 @@ compute warps started and finished it, and when it was published.  The buffer
   [6] compute start  [9] compute end                                  (%globaltimer, ns)
   [7] [8] SM-cycle counts of the task's phases:
       remaining tile: [7] = tile-load wait | chunk waits << 20 | predecessor-tile
-                      wait << 40 (20 bits each), [8] = relaxation end | whole << 32
+                      wait << 40 (20 bits each; the last is 0: those tiles come with
+                      the operands), [8] = relaxation end | whole << 32
                       (type 4: of its tile part)
       pivot / panel:  [7] = operands loaded | relaxed << 32,
                       [8] = results stored | whole << 32
