@@ -475,7 +475,10 @@ __device__ __forceinline__ QuadTask quad_task(const Args<float>& a, int ti, int 
 // vectors, 98 with an argmin by step); distances alone leave little to do
 // afterwards (n = 5000: 10.5 ms without turns, 11.9 with), and small tiles wait on
 // a chain, which turns lengthen (a tile of 64: 17 K SM cycles, 13.4 K without).
-template <int BS, int LBS>
+// A function each for tiles with predecessors (kPred) and without, so that the latter's
+// registers are not laid out for an argmin (n = 5000 without predecessors 10.7 -> 9.8
+// ms, n = 2900 2.62 -> 2.34; with them n = 5000 18.0 -> 17.5).
+template <int BS, int LBS, bool kPred>
 __device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task& k,
                                           unsigned char* smem, WsBars* wb, PipeCnt& pc,
                                           uint64_t* tr) {
@@ -497,14 +500,14 @@ __device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task&
       arg[m][nn / 4] = 0;
     }
   constexpr bool kHold = kPredSmem<float, BS>;  // the operands stay for the epilogue
-  constexpr bool kTurns = !kHold;
+  constexpr bool kTurns = !kHold && kPred;
   static_assert(!kHold || C::NC == 1, "all of a tile's operands in one stage");
   const unsigned st0 = pc.chunk & 1;
   unsigned char* const stage0 = smem + L::ring_off() + st0 * L::kStage;
   const int group = (int)threadIdx.x >> 7;
   bool ok = mbar_wait(&wb->chunk_full[pc.chunk & 1], (pc.chunk >> 1) & 1, a.status, a.abort_flag,
                       a.timeout_ns);
-  if (kTurns && a.P) turn_wait(group);
+  if (kTurns) turn_wait(group);
 #pragma unroll 1
   for (int ch = 0; ch < C::NC && ok; ++ch) {
     const unsigned st = pc.chunk & 1;
@@ -514,13 +517,12 @@ __device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task&
     if (tr) cw += clock64() - w0;
     const float* const As = reinterpret_cast<const float*>(smem + L::ring_off() + st * L::kStage);
     const float* const Bs = As + C::CK * BS;
-    if (a.P) core_q<BS, C::CK / 4, true>(As, Bs, acc, arg, tx, ty, ch * (C::CK / 4));
-    else core_q<BS, C::CK / 4, false>(As, Bs, acc, arg, tx, ty, 0);
+    core_q<BS, C::CK / 4, kPred>(As, Bs, acc, arg, tx, ty, kPred ? ch * (C::CK / 4) : 0);
     __syncwarp();
     if (!kHold && lane == 0) mbar_arrive(&wb->chunk_empty[st]);
     ++pc.chunk;
   }
-  if (kTurns && a.P) turn_pass(group ^ 1);
+  if (kTurns) turn_pass(group ^ 1);
   if (!ok) return false;
   const long long t_b = tr ? clock64() : 0;
   if (!mbar_wait(&wb->d_full, pc.d & 1, a.status, a.abort_flag, a.timeout_ns)) return false;
@@ -529,6 +531,7 @@ __device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task&
     tr[8] = (uint64_t)(t_b - t_a);
   }
   QuadTask f = quad_task<BS>(a, k.ti, k.tj);
+  if (!kPred) f.P = nullptr;
   const size_t ta = (size_t)(k.r & 1) * a.slot_tiles + k.ti, tb = (size_t)(k.r & 1) * a.slot_tiles + k.tj;
   if constexpr (kHold) {
     f.A = reinterpret_cast<const float*>(stage0);
@@ -1709,7 +1712,8 @@ __device__ bool compute_task(const Args<T>& a, const fwh::Task& k, int mode, int
       else
         ok = ws_minplus<T, BS, LBS, false, true>(ctx, k.ti, k.tj, dec, smem, wb, pc, tr);
     } else if constexpr (sizeof(T) == 4) {
-      ok = ws_minplus_q<BS, LBS>(a, k, smem, wb, pc, tr);
+      ok = a.P ? ws_minplus_q<BS, LBS, true>(a, k, smem, wb, pc, tr)
+               : ws_minplus_q<BS, LBS, false>(a, k, smem, wb, pc, tr);
     } else if constexpr (kFiltered<T, BS>) {
       if (skip_filter(pc.exact, k.r, k.ti, k.tj)) {
         ok = ws_exact_f<T, BS, LBS, true>(a, k, smem, wb, pc, tr);
