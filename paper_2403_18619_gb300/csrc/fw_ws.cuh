@@ -475,9 +475,10 @@ __device__ __forceinline__ QuadTask quad_task(const Args<float>& a, int ti, int 
 // vectors, 98 with an argmin by step); distances alone leave little to do
 // afterwards (n = 5000: 10.5 ms without turns, 11.9 with), and small tiles wait on
 // a chain, which turns lengthen (a tile of 64: 17 K SM cycles, 13.4 K without).
-// A function each for tiles with predecessors (kPred) and without, so that the latter's
-// registers are not laid out for an argmin (n = 5000 without predecessors 10.7 -> 9.8
-// ms, n = 2900 2.62 -> 2.34; with them n = 5000 18.0 -> 17.5).
+// A function each for tiles with predecessors (kPred) and without: as one, the tile of
+// 128 reloads 264 bytes of spilled registers, apart 224 with predecessors and 8 without
+// (n = 5000 without predecessors 10.7 -> 9.8 ms, with them 18.0 -> 17.5).  Tiles of 64
+// spill in neither form and gain too (n = 2900 without 2.62 -> 2.34); why is not known.
 template <int BS, int LBS, bool kPred>
 __device__ __noinline__ bool ws_minplus_q(const Args<float>& a, const fwh::Task& k,
                                           unsigned char* smem, WsBars* wb, PipeCnt& pc,
@@ -689,7 +690,10 @@ __device__ __noinline__ bool ws_panel_q(const Args<float>& a, const fwh::Task& k
   } else {
     f.Psrc = is_row ? snapP : a.pivP + (size_t)(r & 1) * BS * BS;
   }
-  core_q<BS, BS / 4, true>(f.A, f.B, acc, arg, tx, ty, 0);
+  // (No argmin that nobody reads: without predecessors n = 5000 9.8 -> 9.5 ms, n = 2048
+  // 1.13 -> 1.10, n = 2900 2.33 -> 2.33.)
+  if (Pt) core_q<BS, BS / 4, true>(f.A, f.B, acc, arg, tx, ty, 0);
+  else core_q<BS, BS / 4, false>(f.A, f.B, acc, arg, tx, ty, 0);
   finish_tile_q<BS, false, kSmem>(f, own, nrow, ncol, acc, arg, tx, ty,
                                          reinterpret_cast<uint16_t*>(smem + L::scr_off() +
                                                                      (tid >> 5) * L::kScrWarp));
