@@ -472,7 +472,7 @@ __device__ __forceinline__ QuadTask quad_task(const Args<float>& a, int ti, int 
 // relaxations).  Tiles of 128 with predecessors are relaxed in turns, each group of
 // warps with the pipes to itself while the other finds the steps of what it
 // improved (n = 8192: 78 ms, 83 without turns; 73 since distances leave in
-// vectors, 98 with an argmin by step); distances alone leave little to do
+// vectors, 71 in a function of its own, 98 with an argmin by step); distances alone leave little to do
 // afterwards (n = 5000: 10.5 ms without turns, 11.9 with), and small tiles wait on
 // a chain, which turns lengthen (a tile of 64: 17 K SM cycles, 13.4 K without).
 // A function each for tiles with predecessors (kPred) and without: as one, the tile of
